@@ -537,8 +537,9 @@ int loip_k_pack(const uint16_t* in, uint64_t n_sb, uint8_t* out, uint32_t* raw_l
                 uint32_t raw_cap, void* stream);
 int loip_k_unpack(const uint8_t* in, uint64_t n_sb, uint16_t* out, void* stream);
 
-/* 0 if no tensor-core GEMM launch has recorded a failure (a bounded pipeline
- * wait that ran out); otherwise the first failure code.  -1 if unreadable. */
+/* 0 if no tensor-core GEMM or batched projection launch has recorded a failure
+ * (a bounded pipeline wait that ran out); otherwise the first failure code.
+ * -1 if unreadable. */
 int loip_k_tc_status(void);
 
 /* Final RMSNorm and LM head: z = RMSNorm(x) * g_final (fp32 [B, H], may be

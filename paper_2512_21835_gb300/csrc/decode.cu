@@ -15,8 +15,7 @@
 #include <math.h>
 #include <stdint.h>
 
-#include <utility>
-
+#include "gemv.cuh"
 #include "internal.h"
 
 namespace loip {
@@ -27,10 +26,10 @@ constexpr int kThreads = kWarps * 32;
 constexpr int kStageFloats = 16384;  // 64 KB of staged activations per block
 constexpr int kMaxChunks = 256;      // pages per request in split attention (16384 positions)
 #ifndef LOIP_GEMV_MIN_BLOCKS1
-#define LOIP_GEMV_MIN_BLOCKS1 2  // resident blocks per SM the registers are sized for, batch tile 1
+#define LOIP_GEMV_MIN_BLOCKS1 2  // resident blocks per SM the registers are sized for
 #endif
 #ifndef LOIP_GEMV_JU1
-#define LOIP_GEMV_JU1 4  // 128-bit loads per row and batch at batch tile 1
+#define LOIP_GEMV_JU1 4  // 128-bit loads per row and batch
 #endif
 
 __device__ __forceinline__ uint4 ld_stream(const uint16_t* p) {
@@ -40,16 +39,6 @@ __device__ __forceinline__ uint4 ld_stream(const uint16_t* p) {
         : "l"(p));
     return r;
 }
-__device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
-__device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
-__device__ __forceinline__ float bf2f(uint16_t h) { return __uint_as_float((uint32_t)h << 16); }
-__device__ __forceinline__ uint16_t f2bf(float f) { return __bfloat16_as_ushort(__float2bfloat16_rn(f)); }
-
-// Programmatic dependent launch: let the next kernel of the stream start its
-// independent prologue, and wait for the previous kernel's results.  Both are
-// no-ops for a kernel launched without the attribute.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
@@ -65,48 +54,9 @@ __device__ __forceinline__ float warp_max(float v) {
     return v;
 }
 
-// Orderable 64-bit argmax key: larger value wins; on equal values the lower
-// index wins (the low word stores ~index).
-__device__ __forceinline__ uint64_t argmax_key(float v, uint32_t idx) {
-    uint32_t u = __float_as_uint(v);
-    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-    return ((uint64_t)u << 32) | (uint64_t)(0xffffffffu - idx);
-}
-
-__device__ __forceinline__ char* kv_row(const KvView& kv, int req, int pos, int kv_or_v, int head, int Hkv, int d) {
-    int page = pos / kv.page_tokens, t = pos - page * kv.page_tokens;
-    char* p = kv.base + kv.page_offsets[(int64_t)req * kv.max_pages + page] + (uint64_t)kv.layer * kv.layer_page_bytes;
-    p += ((uint64_t)(kv_or_v * Hkv + head) * kv.page_tokens + t) * (uint64_t)d * 2u;
-    return p;
-}
-
 // ----------------------------------------------------------------------------
 // Matrix-vector family
 // ----------------------------------------------------------------------------
-enum { EPI_QKV = 0, EPI_RESID = 1, EPI_SWIGLU = 2, EPI_LOGITS = 3 };
-
-struct GemvParams {
-    const float* in;     // [B, K] fp32 activations
-    const uint16_t* g;   // [K] gain: input is RMSNorm(in) * g when non-null
-    const uint16_t* w0;  // [N, K]
-    const uint16_t* w1;  // [N, K] (SwiGLU up projection)
-    int B, K, N, n_units;
-    float eps;
-    float* out;
-    float* z;
-    uint64_t* keys;
-    // QKV epilogue
-    int Hq, Hkv, d;
-    const int32_t* positions;
-    const int32_t* row_req;
-    KvView kv;
-    RopeFreqs rope;
-    int w_host;  // weights are read in place from mapped host memory: no L2 prefetch of them
-    float* qk_raw;  // QK-norm models: query/key rows leave unrotated here ([B][(Hq + 2 Hkv) d])
-    int pf_stride;  // block-tile kernel, > 0: before its dependency wait, block b pulls tiles
-                    // b + pf_stride, b + 2 pf_stride, ... (the later waves) into L2
-};
-
 // rows handled per warp unit, by epilogue
 template <int EPI>
 struct UnitRows {
@@ -130,61 +80,36 @@ __device__ __forceinline__ const uint16_t* unit_row(const GemvParams& p, int uni
     }
 }
 
-// Staged-activation index of element k of row b inside a chunk.
-template <int BT>
-__device__ __forceinline__ int stage_index(int k, int b) {
-    int j = k >> 8, lane = (k >> 3) & 31;
-    if (BT == 1) {
-        int half = (k >> 2) & 1, e4 = k & 3;
-        return ((j * 2 + half) * 32 + lane) * 4 + e4;
-    } else {
-        int e = k & 7;
-        return ((j * 8 + e) * BT + b) * 32 + lane;
-    }
+// Staged-activation index of element k inside a chunk.
+__device__ __forceinline__ int stage_index(int k) {
+    const int j = k >> 8, lane = (k >> 3) & 31, half = (k >> 2) & 1, e4 = k & 3;
+    return ((j * 2 + half) * 32 + lane) * 4 + e4;
 }
 
-template <int BT, int U>
-__device__ __forceinline__ void fma_block(float (&acc)[U][BT], const uint4 (&w)[U], const float* __restrict__ s,
-                                          int j, int lane) {
-    if (BT == 1) {
-        const float4* s4 = reinterpret_cast<const float4*>(s);
-        float4 ya = s4[(j * 2) * 32 + lane], yb = s4[(j * 2 + 1) * 32 + lane];
+template <int U>
+__device__ __forceinline__ void fma_block(float (&acc)[U], const uint4 (&w)[U], const float* __restrict__ s, int j,
+                                          int lane) {
+    const float4* s4 = reinterpret_cast<const float4*>(s);
+    float4 ya = s4[(j * 2) * 32 + lane], yb = s4[(j * 2 + 1) * 32 + lane];
 #pragma unroll
-        for (int r = 0; r < U; ++r) {
-            float a = acc[r][0];
-            a = fmaf(bf_lo(w[r].x), ya.x, a);
-            a = fmaf(bf_hi(w[r].x), ya.y, a);
-            a = fmaf(bf_lo(w[r].y), ya.z, a);
-            a = fmaf(bf_hi(w[r].y), ya.w, a);
-            a = fmaf(bf_lo(w[r].z), yb.x, a);
-            a = fmaf(bf_hi(w[r].z), yb.y, a);
-            a = fmaf(bf_lo(w[r].w), yb.z, a);
-            a = fmaf(bf_hi(w[r].w), yb.w, a);
-            acc[r][0] = a;
-        }
-    } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            float wf[U];
-#pragma unroll
-            for (int r = 0; r < U; ++r) {
-                uint32_t word = (e < 2) ? w[r].x : (e < 4) ? w[r].y : (e < 6) ? w[r].z : w[r].w;
-                wf[r] = (e & 1) ? bf_hi(word) : bf_lo(word);
-            }
-#pragma unroll
-            for (int b = 0; b < BT; ++b) {
-                float y = s[((j * 8 + e) * BT + b) * 32 + lane];
-#pragma unroll
-                for (int r = 0; r < U; ++r) acc[r][b] = fmaf(wf[r], y, acc[r][b]);
-            }
-        }
+    for (int r = 0; r < U; ++r) {
+        float a = acc[r];
+        a = fmaf(bf_lo(w[r].x), ya.x, a);
+        a = fmaf(bf_hi(w[r].x), ya.y, a);
+        a = fmaf(bf_lo(w[r].y), ya.z, a);
+        a = fmaf(bf_hi(w[r].y), ya.w, a);
+        a = fmaf(bf_lo(w[r].z), yb.x, a);
+        a = fmaf(bf_hi(w[r].z), yb.y, a);
+        a = fmaf(bf_lo(w[r].w), yb.z, a);
+        a = fmaf(bf_hi(w[r].w), yb.w, a);
+        acc[r] = a;
     }
 }
 
 // Accumulates the unit's rows over staged chunk [kc0, kc0 + kn).  Two register
 // batches of JU 128-bit loads per row alternate, so the next batch is in flight
 // while the current one is consumed.
-template <int BT, int U, int JU>
+template <int U, int JU>
 __device__ __forceinline__ void load_batch(uint4 (&w)[JU][U], const uint16_t* const (&rp)[U], const bool (&rv)[U],
                                            int kc0, int j0, int nj, int K, int lane) {
 #pragma unroll
@@ -198,119 +123,104 @@ __device__ __forceinline__ void load_batch(uint4 (&w)[JU][U], const uint16_t* co
 
 // Loads per row and batch: a warp keeps about 2 x 8 x 16 bytes per lane in
 // flight whatever its unit's row count.
-template <int BT, int U>
+template <int U>
 struct Batch {
-    static constexpr int JU = (BT == 1) ? (U == 1 ? 2 * LOIP_GEMV_JU1 : LOIP_GEMV_JU1) : (BT == 2) ? 4 : 2;
+    static constexpr int JU = U == 1 ? 2 * LOIP_GEMV_JU1 : LOIP_GEMV_JU1;
 };
 
-template <int BT, int U, int EPI>
-__device__ __forceinline__ void unit_chunk(float (&acc)[U][BT], const uint16_t* const (&rp)[U], const bool (&rv)[U],
+template <int U>
+__device__ __forceinline__ void unit_chunk(float (&acc)[U], const uint16_t* const (&rp)[U], const bool (&rv)[U],
                                            const float* __restrict__ s, int kc0, int kn, int K, int lane) {
-    constexpr int JU = Batch<BT, U>::JU;
+    constexpr int JU = Batch<U>::JU;
     const int nj = (kn + 255) >> 8;
     uint4 wa[JU][U], wb[JU][U];
-    load_batch<BT, U, JU>(wa, rp, rv, kc0, 0, nj, K, lane);
+    load_batch<U, JU>(wa, rp, rv, kc0, 0, nj, K, lane);
     for (int j0 = 0; j0 < nj; j0 += 2 * JU) {
-        load_batch<BT, U, JU>(wb, rp, rv, kc0, j0 + JU, nj, K, lane);
+        load_batch<U, JU>(wb, rp, rv, kc0, j0 + JU, nj, K, lane);
 #pragma unroll
         for (int jj = 0; jj < JU; ++jj)
-            if (j0 + jj < nj) fma_block<BT, U>(acc, wa[jj], s, j0 + jj, lane);
-        load_batch<BT, U, JU>(wa, rp, rv, kc0, j0 + 2 * JU, nj, K, lane);
+            if (j0 + jj < nj) fma_block<U>(acc, wa[jj], s, j0 + jj, lane);
+        load_batch<U, JU>(wa, rp, rv, kc0, j0 + 2 * JU, nj, K, lane);
 #pragma unroll
         for (int jj = 0; jj < JU; ++jj)
-            if (j0 + JU + jj < nj) fma_block<BT, U>(acc, wb[jj], s, j0 + JU + jj, lane);
+            if (j0 + JU + jj < nj) fma_block<U>(acc, wb[jj], s, j0 + JU + jj, lane);
     }
 }
 
-template <int BT, int U, int EPI>
-__device__ __forceinline__ void unit_epilogue(const GemvParams& p, int unit, float (&acc)[U][BT], const float* inv,
-                                              int lane, uint64_t (&best)[BT]) {
+template <int U, int EPI>
+__device__ __forceinline__ void unit_epilogue(const GemvParams& p, int unit, float (&acc)[U], float inv, int lane,
+                                              uint64_t& best) {
 #pragma unroll
-    for (int r = 0; r < U; ++r)
-#pragma unroll
-        for (int b = 0; b < BT; ++b) acc[r][b] = warp_sum(acc[r][b]);
+    for (int r = 0; r < U; ++r) acc[r] = warp_sum(acc[r]);
     if (EPI == EPI_QKV) {
-        if (unit >= p.n_units) return;
+        if (unit >= p.n_units || lane != 0) return;
         const int half = p.d >> 1;
         const int h = unit / half, i = unit - h * half;
-#pragma unroll
-        for (int b = 0; b < BT; ++b) {
-            if (lane != b || b >= p.B) continue;
-            float v0 = acc[0][b] * inv[b], v1 = acc[1][b] * inv[b];
-            const int pos = p.positions[b];
-            if (p.qk_raw && h < p.Hq + p.Hkv) {  // normalised and rotated by qk_norm_rope_kernel
-                float* raw = p.qk_raw + (size_t)b * (p.Hq + 2 * p.Hkv) * p.d + (size_t)h * p.d;
-                raw[i] = v0;
-                raw[i + half] = v1;
-                continue;
-            }
-            if (h < p.Hq + p.Hkv) {
-                float cf, sf;
-                rope_cos_sin(pos, p.rope.inv_freq[i], &cf, &sf);
-                float r0 = v0 * cf - v1 * sf, r1 = v1 * cf + v0 * sf;
-                v0 = r0;
-                v1 = r1;
-            }
-            if (h < p.Hq) {
-                float* q = p.out + (size_t)b * p.Hq * p.d + (size_t)h * p.d;
-                q[i] = v0;
-                q[i + half] = v1;
-            } else {
-                const int req = p.row_req ? p.row_req[b] : b;
-                const bool is_v = h >= p.Hq + p.Hkv;
-                const int kh = h - p.Hq - (is_v ? p.Hkv : 0);
-                uint16_t* row = reinterpret_cast<uint16_t*>(kv_row(p.kv, req, pos, is_v ? 1 : 0, kh, p.Hkv, p.d));
-                row[i] = f2bf(v0);
-                row[i + half] = f2bf(v1);
-            }
+        float v0 = acc[0] * inv, v1 = acc[1] * inv;
+        const int pos = p.positions[0];
+        if (p.qk_raw && h < p.Hq + p.Hkv) {  // normalised and rotated by qk_norm_rope_kernel
+            float* raw = p.qk_raw + (size_t)h * p.d;
+            raw[i] = v0;
+            raw[i + half] = v1;
+            return;
+        }
+        if (h < p.Hq + p.Hkv) {
+            float cf, sf;
+            rope_cos_sin(pos, p.rope.inv_freq[i], &cf, &sf);
+            float r0 = v0 * cf - v1 * sf, r1 = v1 * cf + v0 * sf;
+            v0 = r0;
+            v1 = r1;
+        }
+        if (h < p.Hq) {
+            float* q = p.out + (size_t)h * p.d;
+            q[i] = v0;
+            q[i + half] = v1;
+        } else {
+            const int req = p.row_req ? p.row_req[0] : 0;
+            const bool is_v = h >= p.Hq + p.Hkv;
+            const int kh = h - p.Hq - (is_v ? p.Hkv : 0);
+            uint16_t* row = reinterpret_cast<uint16_t*>(kv_row(p.kv, req, pos, is_v ? 1 : 0, kh, p.Hkv, p.d));
+            row[i] = f2bf(v0);
+            row[i + half] = f2bf(v1);
         }
     } else if (EPI == EPI_RESID) {
 #pragma unroll
-        for (int r = 0; r < U; ++r)
-#pragma unroll
-            for (int b = 0; b < BT; ++b) {
-                int row = unit * U + r;
-                if (lane == r * BT + b && b < p.B && row < p.N) p.out[(size_t)b * p.N + row] += acc[r][b];
-            }
-    } else if (EPI == EPI_SWIGLU) {
-        if (unit >= p.n_units) return;
-#pragma unroll
-        for (int b = 0; b < BT; ++b) {
-            if (lane != b || b >= p.B) continue;
-            float gt = acc[0][b] * inv[b], ut = acc[1][b] * inv[b];
-            float silu = gt / (1.0f + expf(-gt));
-            p.out[(size_t)b * p.N + unit] = silu * ut;
+        for (int r = 0; r < U; ++r) {
+            int row = unit * U + r;
+            if (lane == r && row < p.N) p.out[row] += acc[r];
         }
+    } else if (EPI == EPI_SWIGLU) {
+        if (unit >= p.n_units || lane != 0) return;
+        float gt = acc[0] * inv, ut = acc[1] * inv;
+        float silu = gt / (1.0f + expf(-gt));
+        p.out[unit] = silu * ut;
     } else {  // EPI_LOGITS
 #pragma unroll
         for (int r = 0; r < U; ++r) {
             int row = unit * U + r;
             if (row >= p.N) continue;
-#pragma unroll
-            for (int b = 0; b < BT; ++b) {
-                if (b >= p.B) continue;
-                float v = acc[r][b] * inv[b];
-                if (p.out && lane == r * BT + b) p.out[(size_t)b * p.N + row] = v;
-                uint64_t key = argmax_key(v, (uint32_t)row);
-                best[b] = key > best[b] ? key : best[b];
-            }
+            float v = acc[r] * inv;
+            if (p.out && lane == r) p.out[row] = v;
+            uint64_t key = argmax_key(v, (uint32_t)row);
+            best = key > best ? key : best;
         }
     }
 }
 
-template <int BT, int EPI>
-__global__ void __launch_bounds__(kThreads, BT == 1 ? LOIP_GEMV_MIN_BLOCKS1 : 2) gemv_kernel(GemvParams p) {
+// Batch 1, row-rich matrices and weights in mapped host memory (gemv_batch.cu
+// serves larger batches).
+template <int EPI>
+__global__ void __launch_bounds__(kThreads, LOIP_GEMV_MIN_BLOCKS1) gemv_kernel(GemvParams p) {
     constexpr int U = UnitRows<EPI>::U;
     extern __shared__ __align__(16) float s_stage[];
-    __shared__ float s_red[kWarps][BT];
-    __shared__ float s_inv[BT];
-    __shared__ uint64_t s_keys[kWarps][BT];
+    __shared__ float s_red[kWarps];
+    __shared__ float s_inv;
+    __shared__ uint64_t s_keys[kWarps];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int K = p.K;
-    int kc_max = (kStageFloats / BT) & ~255;
-    const bool single = K <= kc_max;
-    const int KC = single ? ((K + 255) & ~255) : kc_max;
+    const bool single = K <= kStageFloats;
+    const int KC = single ? ((K + 255) & ~255) : kStageFloats;
     const bool norm = p.g != nullptr;
 
     // weights never depend on the previous kernel: start pulling this warp's
@@ -327,75 +237,57 @@ __global__ void __launch_bounds__(kThreads, BT == 1 ? LOIP_GEMV_MIN_BLOCKS1 : 2)
     }
     pdl_wait();
 
-    float ss[BT];
-#pragma unroll
-    for (int b = 0; b < BT; ++b) ss[b] = 0.f;
-    uint64_t best[BT];
-#pragma unroll
-    for (int b = 0; b < BT; ++b) best[b] = 0;
+    float ss = 0.f;
+    uint64_t best = 0;
 
-    // Stages chunk [kc0, kc0 + KC) of every activation row: 16-byte loads, four
+    // Stages chunk [kc0, kc0 + KC) of the activation row: 16-byte loads, four
     // per thread issued before any is consumed, so one L2 round trip covers
     // 4 x 256 x 16 bytes; zeros pad the chunk to a multiple of 256 elements.
     auto stage = [&](int kc0) {
         const int kn = min(KC, K - kc0), kpad = (kn + 255) & ~255;
         const int n4 = kpad >> 2;
         constexpr int UN = 4;
+        for (int base = tid; base < n4; base += kThreads * UN) {
+            float4 v[UN];
+            uint2 gv[UN];
 #pragma unroll
-        for (int b = 0; b < BT; ++b) {
-            for (int base = tid; base < n4; base += kThreads * UN) {
-                float4 v[UN];
-                uint2 gv[UN];
+            for (int u = 0; u < UN; ++u) {
+                const int k = (base + u * kThreads) * 4;
+                const bool ok = k < kn;
+                v[u] = ok ? *reinterpret_cast<const float4*>(p.in + kc0 + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+                gv[u] = (ok && norm) ? *reinterpret_cast<const uint2*>(p.g + kc0 + k) : make_uint2(0, 0);
+            }
 #pragma unroll
-                for (int u = 0; u < UN; ++u) {
-                    const int k = (base + u * kThreads) * 4;
-                    const bool ok = k < kn && b < p.B;
-                    v[u] = ok ? *reinterpret_cast<const float4*>(p.in + (size_t)b * K + kc0 + k)
-                              : make_float4(0.f, 0.f, 0.f, 0.f);
-                    gv[u] = (ok && norm) ? *reinterpret_cast<const uint2*>(p.g + kc0 + k) : make_uint2(0, 0);
+            for (int u = 0; u < UN; ++u) {
+                const int k = (base + u * kThreads) * 4;
+                if (k >= kpad) continue;
+                float4 w = v[u];
+                if (norm) {
+                    ss = fmaf(w.x, w.x, ss);
+                    ss = fmaf(w.y, w.y, ss);
+                    ss = fmaf(w.z, w.z, ss);
+                    ss = fmaf(w.w, w.w, ss);
+                    w.x *= bf_lo(gv[u].x);
+                    w.y *= bf_hi(gv[u].x);
+                    w.z *= bf_lo(gv[u].y);
+                    w.w *= bf_hi(gv[u].y);
                 }
-#pragma unroll
-                for (int u = 0; u < UN; ++u) {
-                    const int k = (base + u * kThreads) * 4;
-                    if (k >= kpad) continue;
-                    float4 w = v[u];
-                    if (norm) {
-                        ss[b] = fmaf(w.x, w.x, ss[b]);
-                        ss[b] = fmaf(w.y, w.y, ss[b]);
-                        ss[b] = fmaf(w.z, w.z, ss[b]);
-                        ss[b] = fmaf(w.w, w.w, ss[b]);
-                        w.x *= bf_lo(gv[u].x);
-                        w.y *= bf_hi(gv[u].x);
-                        w.z *= bf_lo(gv[u].y);
-                        w.w *= bf_hi(gv[u].y);
-                    }
-                    if (BT == 1) {
-                        *reinterpret_cast<float4*>(&s_stage[stage_index<1>(k, 0)]) = w;
-                    } else {
-                        s_stage[stage_index<BT>(k, b)] = w.x;
-                        s_stage[stage_index<BT>(k + 1, b)] = w.y;
-                        s_stage[stage_index<BT>(k + 2, b)] = w.z;
-                        s_stage[stage_index<BT>(k + 3, b)] = w.w;
-                    }
-                }
+                *reinterpret_cast<float4*>(&s_stage[stage_index(k)]) = w;
             }
         }
     };
     auto finish_norm = [&]() {
         if (norm) {
-#pragma unroll
-            for (int b = 0; b < BT; ++b) {
-                float t = warp_sum(ss[b]);
-                if (lane == 0) s_red[warp][b] = t;
-            }
+            const float t = warp_sum(ss);
+            if (lane == 0) s_red[warp] = t;
             __syncthreads();
-            if (tid < BT) {
+            if (tid == 0) {
                 float t = 0.f;
-                for (int w = 0; w < kWarps; ++w) t += s_red[w][tid];
-                s_inv[tid] = 1.0f / sqrtf(t / (float)K + p.eps);
+                for (int w = 0; w < kWarps; ++w) t += s_red[w];
+                s_inv = 1.0f / sqrtf(t / (float)K + p.eps);
             }
-        } else if (tid < BT) {
-            s_inv[tid] = 1.0f;
+        } else if (tid == 0) {
+            s_inv = 1.0f;
         }
         __syncthreads();
     };
@@ -404,21 +296,17 @@ __global__ void __launch_bounds__(kThreads, BT == 1 ? LOIP_GEMV_MIN_BLOCKS1 : 2)
         stage(0);
         __syncthreads();
         finish_norm();
-        float inv[BT];
-#pragma unroll
-        for (int b = 0; b < BT; ++b) inv[b] = s_inv[b];
+        const float inv = s_inv;
         for (int unit = blockIdx.x * kWarps + warp; unit < p.n_units; unit += gridDim.x * kWarps) {
             const uint16_t* rp[U];
             bool rv[U];
 #pragma unroll
             for (int r = 0; r < U; ++r) rp[r] = unit_row<EPI>(p, unit, r, rv[r]);
-            float acc[U][BT];
+            float acc[U];
 #pragma unroll
-            for (int r = 0; r < U; ++r)
-#pragma unroll
-                for (int b = 0; b < BT; ++b) acc[r][b] = 0.f;
-            unit_chunk<BT, U, EPI>(acc, rp, rv, s_stage, 0, K, K, lane);
-            unit_epilogue<BT, U, EPI>(p, unit, acc, inv, lane, best);
+            for (int r = 0; r < U; ++r) acc[r] = 0.f;
+            unit_chunk<U>(acc, rp, rv, s_stage, 0, K, K, lane);
+            unit_epilogue<U, EPI>(p, unit, acc, inv, lane, best);
         }
     } else {
         const int unit = blockIdx.x * kWarps + warp;
@@ -426,40 +314,30 @@ __global__ void __launch_bounds__(kThreads, BT == 1 ? LOIP_GEMV_MIN_BLOCKS1 : 2)
         bool rv[U];
 #pragma unroll
         for (int r = 0; r < U; ++r) rp[r] = unit_row<EPI>(p, unit, r, rv[r]);
-        float acc[U][BT];
+        float acc[U];
 #pragma unroll
-        for (int r = 0; r < U; ++r)
-#pragma unroll
-            for (int b = 0; b < BT; ++b) acc[r][b] = 0.f;
+        for (int r = 0; r < U; ++r) acc[r] = 0.f;
         for (int kc0 = 0; kc0 < K; kc0 += KC) {
             __syncthreads();
             stage(kc0);
             __syncthreads();
-            unit_chunk<BT, U, EPI>(acc, rp, rv, s_stage, kc0, min(KC, K - kc0), K, lane);
+            unit_chunk<U>(acc, rp, rv, s_stage, kc0, min(KC, K - kc0), K, lane);
         }
         finish_norm();
-        float inv[BT];
-#pragma unroll
-        for (int b = 0; b < BT; ++b) inv[b] = s_inv[b];
-        unit_epilogue<BT, U, EPI>(p, unit, acc, inv, lane, best);
+        unit_epilogue<U, EPI>(p, unit, acc, s_inv, lane, best);
     }
 
     if (EPI == EPI_LOGITS) {
-        if (lane == 0)
-#pragma unroll
-            for (int b = 0; b < BT; ++b) s_keys[warp][b] = best[b];
+        if (lane == 0) s_keys[warp] = best;
         __syncthreads();
-        if (tid < BT) {
+        if (tid == 0) {
             uint64_t k = 0;
-            for (int w = 0; w < kWarps; ++w) k = s_keys[w][tid] > k ? s_keys[w][tid] : k;
-            p.keys[(size_t)blockIdx.x * BT + tid] = k;
+            for (int w = 0; w < kWarps; ++w) k = s_keys[w] > k ? s_keys[w] : k;
+            p.keys[blockIdx.x] = k;
         }
         // final hidden z = RMSNorm(x) * g, written once
-        if (blockIdx.x == 0 && p.z) {
-            for (int b = 0; b < p.B; ++b)
-                for (int k = tid; k < K; k += kThreads)
-                    p.z[(size_t)b * K + k] = p.in[(size_t)b * K + k] * s_inv[b] * bf2f(p.g[k]);
-        }
+        if (blockIdx.x == 0 && p.z)
+            for (int k = tid; k < K; k += kThreads) p.z[k] = p.in[k] * s_inv * bf2f(p.g[k]);
     }
 }
 
@@ -734,24 +612,6 @@ __global__ void argmax_reduce_kernel(const uint64_t* keys, int nblocks, int BT, 
     if (threadIdx.x == 0 && b < B) tokens[b] = (int32_t)(0xffffffffu - (uint32_t)(s[0] & 0xffffffffu));
 }
 
-// Launch with programmatic stream serialisation when `pdl` (the previous
-// operation on the stream is a kernel of the same chain).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl,
-                     Args&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = pdl ? at : nullptr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
 template <int EPI>
 cudaError_t launch_gemv(GemvParams& p, cudaStream_t st, bool pdl, int* nblocks_out = nullptr) {
     // Batch 1: matrices with few rows (QKV, O-proj, down) keep too few units per
@@ -762,6 +622,7 @@ cudaError_t launch_gemv(GemvParams& p, cudaStream_t st, bool pdl, int* nblocks_o
     // mapped host memory always go to the persistent kernel: over the host link
     // a tile's serial chunk loads along a long row (down, K = 28672) ran at
     // 183 GB/s against the link's 211, which the persistent kernel reaches.
+    if (p.B > 1) return launch_gemv_batch(EPI, p, st, pdl, nblocks_out);  // tensor cores: gemv_batch.cu
     const int rows = (EPI == EPI_SWIGLU) ? 2 * p.n_units : p.N;
     if (p.B == 1 && !p.w_host && rows <= (EPI == EPI_QKV ? 8192 : 16384)) {
         const int per_tile = (EPI == EPI_QKV || EPI == EPI_SWIGLU) ? kTileRows / 2 : kTileRows;
@@ -770,42 +631,31 @@ cudaError_t launch_gemv(GemvParams& p, cudaStream_t st, bool pdl, int* nblocks_o
         if (nblocks_out) *nblocks_out = tiles;
         return launch_k(gemv_tile_kernel<EPI>, dim3(tiles), dim3(kTileWarps * 32), 0, st, pdl, p);
     }
-    int BT = p.B <= 1 ? 1 : p.B <= 2 ? 2 : p.B <= 4 ? 4 : 8;
-    int kc_max = (kStageFloats / BT) & ~255;
-    bool single = p.K <= kc_max;
-    int KC = single ? ((p.K + 255) & ~255) : kc_max;
-    size_t smem = (size_t)KC * BT * sizeof(float);
+    const bool single = p.K <= kStageFloats;
+    const int KC = single ? ((p.K + 255) & ~255) : kStageFloats;
+    const size_t smem = (size_t)KC * sizeof(float);
     int blocks = (p.n_units + kWarps - 1) / kWarps;
     static bool attr_set = false;
     if (!attr_set) {  // before any occupancy query: the stage is above the 48 KB default
-        int bytes = kStageFloats * (int)sizeof(float);
-        cudaFuncSetAttribute(gemv_kernel<1, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        cudaFuncSetAttribute(gemv_kernel<2, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        cudaFuncSetAttribute(gemv_kernel<4, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        cudaFuncSetAttribute(gemv_kernel<8, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        cudaFuncSetAttribute(gemv_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kStageFloats * (int)sizeof(float));
         attr_set = true;
     }
     if (single) {
-        // resident blocks per SM for this stage size (cached per batch tile and size)
-        static int cache_bt[16], cache_smem[16], cache_val[16], cache_n = 0;
+        // resident blocks per SM for this stage size (cached per size)
+        static int cache_smem[16], cache_val[16], cache_n = 0;
         static int sms = 0;
         int per_sm = 0;
         for (int i = 0; i < cache_n; ++i)
-            if (cache_bt[i] == BT && cache_smem[i] == (int)smem) per_sm = cache_val[i];
+            if (cache_smem[i] == (int)smem) per_sm = cache_val[i];
         if (per_sm == 0) {
             int dev;
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             int v = 0;
-            switch (BT) {
-                case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, gemv_kernel<1, EPI>, kThreads, smem); break;
-                case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, gemv_kernel<2, EPI>, kThreads, smem); break;
-                case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, gemv_kernel<4, EPI>, kThreads, smem); break;
-                default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, gemv_kernel<8, EPI>, kThreads, smem); break;
-            }
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, gemv_kernel<EPI>, kThreads, smem);
             per_sm = v < 1 ? 1 : v;
             if (cache_n < 16) {
-                cache_bt[cache_n] = BT;
                 cache_smem[cache_n] = (int)smem;
                 cache_val[cache_n] = per_sm;
                 ++cache_n;
@@ -816,13 +666,7 @@ cudaError_t launch_gemv(GemvParams& p, cudaStream_t st, bool pdl, int* nblocks_o
     }
     if (blocks < 1) blocks = 1;
     if (nblocks_out) *nblocks_out = blocks;
-
-    switch (BT) {
-        case 1: return launch_k(gemv_kernel<1, EPI>, dim3(blocks), dim3(kThreads), smem, st, pdl, p);
-        case 2: return launch_k(gemv_kernel<2, EPI>, dim3(blocks), dim3(kThreads), smem, st, pdl, p);
-        case 4: return launch_k(gemv_kernel<4, EPI>, dim3(blocks), dim3(kThreads), smem, st, pdl, p);
-        default: return launch_k(gemv_kernel<8, EPI>, dim3(blocks), dim3(kThreads), smem, st, pdl, p);
-    }
+    return launch_k(gemv_kernel<EPI>, dim3(blocks), dim3(kThreads), smem, st, pdl, p);
 }
 
 // ----------------------------------------------------------------------------
@@ -2007,7 +1851,7 @@ cudaError_t launch_lm_head(const float* x, const uint16_t* g, const uint16_t* w,
     p.B = B;
     p.K = H;
     p.N = V;
-    p.n_units = (V + 1) / 2;
+    p.n_units = B > 1 ? V : (V + 1) / 2;  // rows, or the row pairs of the batch-1 kernel
     p.eps = eps;
     p.out = logits;
     p.z = z;
@@ -2015,7 +1859,7 @@ cudaError_t launch_lm_head(const float* x, const uint16_t* g, const uint16_t* w,
     int nblocks = 0;
     cudaError_t e = launch_gemv<EPI_LOGITS>(p, st, pdl, &nblocks);
     if (e != cudaSuccess) return e;
-    int BT = B <= 1 ? 1 : B <= 2 ? 2 : B <= 4 ? 4 : 8;
+    const int BT = B > 1 ? 8 : 1;  // keys per block
     return launch_k(argmax_reduce_kernel, dim3(B), dim3(256), 0, st, true, (const uint64_t*)p.keys, nblocks, BT, B,
                     tokens);
 }

@@ -68,6 +68,10 @@ cudaError_t launch_lm_head(const float* x, const uint16_t* g, const uint16_t* w,
                            float* z, float* logits, int32_t* tokens, void* scratch, cudaStream_t st,
                            bool pdl = false);
 size_t lm_head_scratch_bytes(int B, int V);
+// First failure code recorded by a product of 2 to 8 rows (gemv_batch.cu; a
+// bounded pipeline wait that ran out; 0 = none), and the device address of it.
+cudaError_t gemv_batch_error(int* code);
+cudaError_t gemv_batch_error_word(const int** dev);
 
 // Grouped-query attention over the paged cache.  Rows b = 0..B-1 attend over
 // their first ctx_lens[b] positions with query q[b] (ctx_lens NULL: over

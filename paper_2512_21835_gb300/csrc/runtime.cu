@@ -273,6 +273,7 @@ struct loip_ctx {
     cudaEvent_t stage_done[kStages] = {};         // last copy out of the buffer
     int32_t* h_stage = nullptr;  // pinned staging for small transfers (last word: layer-run error)
     bool run_launched = false;   // a layer-run kernel has been enqueued (its error word is checked)
+    const int* gemv_error = nullptr;  // the batched products' error word (device), checked like it
     size_t h_stage_ints = 0;
     int64_t* h_pt = nullptr;     // pinned page-table staging
     // streams and events
@@ -714,11 +715,15 @@ struct loip_ctx {
 
     // After a host sync point: a layer-run kernel whose grid barrier timed out
     // left its error word set; the context cannot continue.
+    // The batched products' pipeline waits are bounded in the same way.
     int check_run_error() {
-        if (!run_launched) return LOIP_OK;
-        if (h_stage[h_stage_ints - 1] != 0) {
+        if (run_launched && h_stage[h_stage_ints - 1] != 0) {
             failed = true;
             return fail(LOIP_ERR_TIMEOUT, "a grid barrier of the persistent layer-run kernel timed out");
+        }
+        if (h_stage[h_stage_ints - 2] != 0) {
+            failed = true;
+            return fail(LOIP_ERR_TIMEOUT, "the weight pipeline of a batched product did not complete");
         }
         return LOIP_OK;
     }
@@ -1844,7 +1849,8 @@ extern "C" int loip_create(const loip_model_desc* desc, const loip_config* cfg_i
                         attention_scratch_floats(cfg.max_batch, c->Hq, c->d, cfg.max_ctx, cfg.page_tokens) * 4,
                         c->compute);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->arena + c->fx.run_sync, 0, 4 * (2 + 4 * kMaxRunLayers), c->compute);
-    c->h_stage[c->h_stage_ints - 1] = 0;
+    c->h_stage[c->h_stage_ints - 1] = c->h_stage[c->h_stage_ints - 2] = 0;
+    if (e == cudaSuccess) e = gemv_batch_error_word(&c->gemv_error);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->compute);
     if (e != cudaSuccess) {
         g_create_error = std::string("CUDA setup failed: ") + cudaGetErrorString(e);
@@ -2130,6 +2136,10 @@ static int decode_step_enqueue(loip_ctx* c, const int32_t* d_tokens, int B, int3
                             cudaMemcpyDeviceToHost, s);
         if (e != cudaSuccess) return c->cuda_fail(e, "error word download");
     }
+    if (B > 1) {
+        e = cudaMemcpyAsync(c->h_stage + c->h_stage_ints - 2, c->gemv_error, 4, cudaMemcpyDeviceToHost, s);
+        if (e != cudaSuccess) return c->cuda_fail(e, "error word download");
+    }
     cudaEventRecord(c->ev_step1, s);
     c->chain = false;
     for (int b = 0; b < B; ++b) c->reqs[b].len += 1;
@@ -2289,7 +2299,11 @@ extern "C" int loip_prefill(loip_ctx* c, const int32_t* tokens, const int32_t* p
     rc = c->wait_event(c->ev_done);
     if (rc) return rc;
     c->collect_kernel_times();
-    int tcerr = 0, aterr = 0;
+    int tcerr = 0, aterr = 0, gverr = 0;
+    if (n_prompts > 1 && (gemv_batch_error(&gverr) != cudaSuccess || gverr != 0)) {
+        c->failed = true;
+        return c->fail(LOIP_ERR_TIMEOUT, "the weight pipeline of a batched product did not complete");
+    }
     if (tc_error(&tcerr) != cudaSuccess || tcerr != 0) {
         c->failed = true;
         return c->fail(LOIP_ERR_TIMEOUT, "tensor-core GEMM pipeline did not complete (code " + std::to_string(tcerr) + ")");
@@ -2630,9 +2644,9 @@ extern "C" int loip_k_unpack(const uint8_t* in, uint64_t n_sb, uint16_t* out, vo
 }
 
 extern "C" int loip_k_tc_status(void) {
-    int code = 0;
-    if (tc_error(&code) != cudaSuccess) return -1;
-    return code;
+    int code = 0, gemv = 0;
+    if (tc_error(&code) != cudaSuccess || gemv_batch_error(&gemv) != cudaSuccess) return -1;
+    return code ? code : gemv;
 }
 
 extern "C" uint64_t loip_k_lm_head_scratch_bytes(int32_t B, int32_t V) {
