@@ -1635,6 +1635,7 @@ struct QkNormParams {
     float* q_out;  // [rows][Hq d]
     KvView kv;
     RopeFreqs rope;
+    const float2* cs;  // rows' rotary table [rows][d/2], or nullptr
 };
 
 // One block of d/2 threads per (row, head): RMSNorm of the head's d values
@@ -1660,7 +1661,13 @@ __global__ void __launch_bounds__(64) qk_norm_rope_kernel(QkNormParams p) {
         v0 = v0 * inv * bf2f(g[i]);
         v1 = v1 * inv * bf2f(g[i + half]);
         float cf, sf;
-        rope_cos_sin(pos, p.rope.inv_freq[i], &cf, &sf);
+        if (p.cs) {
+            const float2 t = p.cs[(size_t)b * half + i];
+            cf = t.x;
+            sf = t.y;
+        } else {
+            rope_cos_sin(pos, p.rope.inv_freq[i], &cf, &sf);
+        }
         const float r0 = v0 * cf - v1 * sf, r1 = v1 * cf + v0 * sf;
         v0 = r0;
         v1 = r1;
@@ -1920,8 +1927,9 @@ cudaError_t launch_attention(const float* q, KvView kv, const int32_t* ctx_lens,
 }
 
 cudaError_t launch_qk_norm_rope(const float* raw, int rows, int Hq, int Hkv, int d, bool with_v, const uint16_t* g_q,
-                                const uint16_t* g_k, float eps, float theta, const int32_t* positions,
-                                const int32_t* row_req, float* q_out, KvView kv, cudaStream_t st, bool pdl) {
+                                const uint16_t* g_k, float eps, float theta, const float2* rope,
+                                const int32_t* positions, const int32_t* row_req, float* q_out, KvView kv,
+                                cudaStream_t st, bool pdl) {
     if (rows < 1 || (d != 64 && d != 128)) return cudaErrorInvalidValue;
     QkNormParams p{};
     p.raw = raw;
@@ -1937,7 +1945,8 @@ cudaError_t launch_qk_norm_rope(const float* raw, int rows, int Hq, int Hkv, int
     p.row_req = row_req;
     p.q_out = q_out;
     p.kv = kv;
-    p.rope = rope_freqs(theta, d);
+    p.cs = rope;
+    if (!rope) p.rope = rope_freqs(theta, d);
     return launch_k(qk_norm_rope_kernel, dim3(Hq + Hkv + (with_v ? Hkv : 0), rows), dim3(d / 2), 0, st, pdl, p);
 }
 

@@ -70,7 +70,7 @@ struct TcParams {
     const int32_t* positions;
     const int32_t* row_req;
     KvView kv;
-    RopeFreqs rope;
+    const float2* rope;  // [M][d/2] (cos, sin) of the rows' positions
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -244,13 +244,16 @@ __device__ __forceinline__ void epi_qkv(const TcParams& p, float (&acc)[128], in
         if (c0 + hc >= p.N) break;  // uniform across the warp
         const int h = (c0 + hc) / D;
         if (h < p.Hq + p.Hkv) {
+            const float4* cs = reinterpret_cast<const float4*>(p.rope + (size_t)row * HALF);
 #pragma unroll
-            for (int i = 0; i < HALF; ++i) {
-                float c, s;
-                rope_cos_sin(pos, p.rope.inv_freq[i], &c, &s);
+            for (int i = 0; i < HALF; i += 2) {
+                const float4 t = cs[i / 2];  // (cos, sin) of i and i + 1
                 const float v0 = acc[hc + i], v1 = acc[hc + HALF + i];
-                acc[hc + i] = v0 * c - v1 * s;
-                acc[hc + HALF + i] = v1 * c + v0 * s;
+                acc[hc + i] = v0 * t.x - v1 * t.y;
+                acc[hc + HALF + i] = v1 * t.x + v0 * t.y;
+                const float w0 = acc[hc + i + 1], w1 = acc[hc + HALF + i + 1];
+                acc[hc + i + 1] = w0 * t.z - w1 * t.w;
+                acc[hc + HALF + i + 1] = w1 * t.z + w0 * t.w;
             }
         }
         if (h < p.Hq) {
@@ -555,8 +558,8 @@ cudaError_t launch_tc(const void* A, bool split, const void* W0, const void* W1,
 }  // namespace
 
 cudaError_t launch_tc_gemm_qkv_rope(const uint16_t* y, bool split, const uint16_t* wqkv, int M, int H, int Hq,
-                                    int Hkv, int d, float theta, const int32_t* positions, const int32_t* row_req,
-                                    float* q, KvView kv, cudaStream_t st) {
+                                    int Hkv, int d, const float2* rope, const int32_t* positions,
+                                    const int32_t* row_req, float* q, KvView kv, cudaStream_t st) {
     if (TBN % d != 0) return cudaErrorInvalidValue;
     TcParams p{};
     p.M = M;
@@ -569,7 +572,7 @@ cudaError_t launch_tc_gemm_qkv_rope(const uint16_t* y, bool split, const uint16_
     p.positions = positions;
     p.row_req = row_req;
     p.kv = kv;
-    p.rope = rope_freqs(theta, d);
+    p.rope = rope;
     return launch_tc<T_QKV>(y, split, wqkv, nullptr, (uint64_t)p.N, p, (p.N + TBN - 1) / TBN, st);
 }
 

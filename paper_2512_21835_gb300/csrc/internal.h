@@ -49,9 +49,11 @@ cudaError_t launch_qkv_rope(const float* x, const uint16_t* g, const uint16_t* w
 // cache), and launch_qk_norm_rope then applies the per-head RMSNorm (gains g_q,
 // g_k [d]) and the rotation and makes the usual stores.  with_v: the value rows
 // of `raw` are copied to the cache as well (prefill, where raw holds all rows).
+// rope: the rows' rotary table (prefill), or nullptr: computed from theta.
 cudaError_t launch_qk_norm_rope(const float* raw, int rows, int Hq, int Hkv, int d, bool with_v, const uint16_t* g_q,
-                                const uint16_t* g_k, float eps, float theta, const int32_t* positions,
-                                const int32_t* row_req, float* q_out, KvView kv, cudaStream_t st, bool pdl = false);
+                                const uint16_t* g_k, float eps, float theta, const float2* rope,
+                                const int32_t* positions, const int32_t* row_req, float* q_out, KvView kv,
+                                cudaStream_t st, bool pdl = false);
 // x += W in (W [N, K] bf16).  prefetch_waves: batch-1 tiles beyond the first
 // wave are pulled into L2 by the first-wave blocks while they wait on the
 // previous kernel (for the O-projection, whose predecessor, attention, leaves
@@ -132,17 +134,27 @@ cudaError_t launch_advance(int32_t* positions, int B, cudaStream_t st, bool pdl 
 cudaError_t launch_generate(uint16_t* out, uint64_t n, uint64_t first, uint64_t seed, uint32_t tensor_id, int kind,
                             cudaStream_t st);
 
+// Cosines and sines of a prefill pass's rows, [M][d/2] (cos, sin): written by
+// the RMSNorm ahead of the QKV projection, read by what rotates its output.
+struct RopeTable {
+    float2* cs;  // nullptr: not wanted
+    const int32_t* positions;
+    int half;  // d / 2
+    RopeFreqs freqs;
+};
 // Prefill (M tokens at once).  y = RMSNorm(x) * g as a split pair of bf16
-// planes [2][M][H]: hi = bf16(y), lo = bf16(y - hi).
+// planes [2][M][H]: hi = bf16(y), lo = bf16(y - hi); with rope.cs set, the rows'
+// rotary table as well.
 cudaError_t launch_rmsnorm_split(const float* x, const uint16_t* g, int M, int H, float eps, uint16_t* y,
-                                 cudaStream_t st);
+                                 const RopeTable& rope, cudaStream_t st);
 // Prefill projections on the tensor cores (tcgen05, TMA), fused epilogues.
 // The activation operand (y, a) is a split pair of bf16 planes [2][M][K] when
 // `split` is set (two MMAs per K step), else one bf16 plane [M][K].  The
-// SwiGLU output `a` is always written as a split pair [2][M][F].
+// SwiGLU output `a` is always written as a split pair [2][M][F].  rope: the
+// rows' rotary table.
 cudaError_t launch_tc_gemm_qkv_rope(const uint16_t* y, bool split, const uint16_t* wqkv, int M, int H, int Hq,
-                                    int Hkv, int d, float theta, const int32_t* positions, const int32_t* row_req,
-                                    float* q, KvView kv, cudaStream_t st);
+                                    int Hkv, int d, const float2* rope, const int32_t* positions,
+                                    const int32_t* row_req, float* q, KvView kv, cudaStream_t st);
 cudaError_t launch_tc_gemm_resid(const uint16_t* a, bool split, const uint16_t* w, int M, int N, int K, float* x,
                                  cudaStream_t st);
 cudaError_t launch_tc_gemm_swiglu(const uint16_t* y, bool split, const uint16_t* wg, const uint16_t* wu, int M, int H,

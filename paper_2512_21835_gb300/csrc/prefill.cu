@@ -17,9 +17,23 @@ namespace {
 __device__ __forceinline__ float bf2f(uint16_t h) { return __uint_as_float((uint32_t)h << 16); }
 __device__ __forceinline__ uint16_t f2bf(float f) { return __bfloat16_as_ushort(__float2bfloat16_rn(f)); }
 
-__global__ void rmsnorm_split_kernel(const float* x, const uint16_t* g, int H, float eps, uint16_t* y) {
+// Row m's entries of the rotary table.  Forming and reducing the angle takes a
+// handful of fp64 operations, and GB300 has few fp64 units: the QKV epilogue,
+// which computed them for every head of a row, spent 48 of its 90 us there (8B,
+// 512 rows).  Once per row and pass, under the row's loads, they cost nothing.
+__device__ __forceinline__ void rope_row(const RopeTable& r, int m) {
+    if (r.cs && (int)threadIdx.x < r.half) {
+        float c, s;
+        rope_cos_sin(r.positions[m], r.freqs.inv_freq[threadIdx.x], &c, &s);
+        r.cs[(size_t)m * r.half + threadIdx.x] = make_float2(c, s);
+    }
+}
+
+__global__ void rmsnorm_split_kernel(const float* x, const uint16_t* g, int H, float eps, uint16_t* y,
+                                     const __grid_constant__ RopeTable rope) {
     __shared__ float red[32];
     const int m = blockIdx.x;
+    rope_row(rope, m);
     const float* xr = x + (size_t)m * H;
     float ss = 0.f;
     for (int k = threadIdx.x; k < H; k += blockDim.x) ss = fmaf(xr[k], xr[k], ss);
@@ -48,7 +62,7 @@ __global__ void rmsnorm_split_kernel(const float* x, const uint16_t* g, int H, f
 // 8-byte stores of four bf16 per plane.  H % 4 == 0, H <= 4 * 256 * kRowVec.
 constexpr int kRowVec = 8;
 __global__ void __launch_bounds__(256) rmsnorm_split_vec_kernel(const float* x, const uint16_t* g, int H, float eps,
-                                                                uint16_t* y) {
+                                                                uint16_t* y, const __grid_constant__ RopeTable rope) {
     __shared__ float red[32];
     __shared__ float4 row4[256 * kRowVec];
     const int m = blockIdx.x, H4 = H >> 2;
@@ -60,6 +74,7 @@ __global__ void __launch_bounds__(256) rmsnorm_split_vec_kernel(const float* x, 
         v[j] = k < H4 ? xr[k] : make_float4(0.f, 0.f, 0.f, 0.f);
         if (k < H4) row4[k] = v[j];
     }
+    rope_row(rope, m);
     __syncthreads();
     const float* row = reinterpret_cast<const float*>(row4);
     float ss = 0.f;
@@ -105,12 +120,12 @@ __global__ void gather_rows_kernel(const float* x, const int32_t* rows, int H, f
 }  // namespace
 
 cudaError_t launch_rmsnorm_split(const float* x, const uint16_t* g, int M, int H, float eps, uint16_t* y,
-                                 cudaStream_t st) {
+                                 const RopeTable& rope, cudaStream_t st) {
     if (M <= 0) return cudaSuccess;
     if (H % 4 == 0 && H <= 4 * 256 * kRowVec && !((uintptr_t)x & 15) && !((uintptr_t)g & 7) && !((uintptr_t)y & 7))
-        rmsnorm_split_vec_kernel<<<M, 256, 0, st>>>(x, g, H, eps, y);
+        rmsnorm_split_vec_kernel<<<M, 256, 0, st>>>(x, g, H, eps, y, rope);
     else
-        rmsnorm_split_kernel<<<M, 256, 0, st>>>(x, g, H, eps, y);
+        rmsnorm_split_kernel<<<M, 256, 0, st>>>(x, g, H, eps, y, rope);
     return cudaGetLastError();
 }
 

@@ -1097,7 +1097,7 @@ struct loip_ctx {
                                             q, kv, nullptr, s, pdl(), host_a, qk_raw);
             if (r == cudaSuccess && qk_raw)
                 r = launch_qk_norm_rope(qk_raw, B, Hq, Hkv, d, false, wa + lay.off_g_q / 2, wa + lay.off_g_k / 2,
-                                        desc.rms_eps, desc.rope_theta, pos_dev, nullptr, q, kv, s, pdl());
+                                        desc.rms_eps, desc.rope_theta, nullptr, pos_dev, nullptr, q, kv, s, pdl());
             return r;
         });
         if (e != cudaSuccess) return cuda_fail(e, "qkv kernel");
@@ -1132,11 +1132,16 @@ struct loip_ctx {
         const int64_t* pt = fixed_ptr<int64_t>(fx.page_table);
         KvView kv = kv_view(l, pt);
         cudaError_t e;
-        e = timed(11, s, [&] { return launch_rmsnorm_split(px, wa + lay.off_g_attn / 2, Mc, H, desc.rms_eps, py, s); });
+        // the rows' rotary table sits in the attention output's buffer until the
+        // attention writes that (4 d of its 4 Hq d bytes per row)
+        RopeTable rope{reinterpret_cast<float2*>(po), pos, d / 2, rope_freqs(desc.rope_theta, d)};
+        e = timed(11, s, [&] {
+            return launch_rmsnorm_split(px, wa + lay.off_g_attn / 2, Mc, H, desc.rms_eps, py, rope, s);
+        });
         if (e == cudaSuccess && !desc.qk_norm)
             e = timed(6, s, [&] {
-                return launch_tc_gemm_qkv_rope(py, true, wa + lay.off_wqkv / 2, Mc, H, Hq, Hkv, d, desc.rope_theta, pos,
-                                               req, pq, kv, s);
+                return launch_tc_gemm_qkv_rope(py, true, wa + lay.off_wqkv / 2, Mc, H, Hq, Hkv, d, rope.cs, pos, req,
+                                               pq, kv, s);
             });
         if (e == cudaSuccess && desc.qk_norm)  // raw projections (GEMM into zeros), then norm + rotation + stores
             e = timed(6, s, [&] {
@@ -1146,7 +1151,7 @@ struct loip_ctx {
                 if (r == cudaSuccess) r = launch_tc_gemm_resid(py, true, wa + lay.off_wqkv / 2, Mc, nqkv, H, raw, s);
                 if (r == cudaSuccess)
                     r = launch_qk_norm_rope(raw, Mc, Hq, Hkv, d, true, wa + lay.off_g_q / 2, wa + lay.off_g_k / 2,
-                                            desc.rms_eps, desc.rope_theta, pos, req, pq, kv, s);
+                                            desc.rms_eps, desc.rope_theta, rope.cs, pos, req, pq, kv, s);
                 return r;
             });
         if (e == cudaSuccess)
@@ -1156,7 +1161,9 @@ struct loip_ctx {
         if (e == cudaSuccess)
             e = timed(8, s, [&] { return launch_tc_gemm_resid(po, true, wa + lay.off_wo / 2, Mc, H, qd, px, s); });
         if (e == cudaSuccess)
-            e = timed(11, s, [&] { return launch_rmsnorm_split(px, wm + lay.off_g_mlp / 2, Mc, H, desc.rms_eps, py, s); });
+            e = timed(11, s, [&] {
+                return launch_rmsnorm_split(px, wm + lay.off_g_mlp / 2, Mc, H, desc.rms_eps, py, RopeTable{}, s);
+            });
         if (e == cudaSuccess)
             e = timed(9, s, [&] {
                 return launch_tc_gemm_swiglu(py, true, wm + lay.off_wg / 2, wm + lay.off_wu / 2, Mc, H, F, pa, s);
