@@ -35,6 +35,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "internal.h"
 
 namespace loip {
@@ -61,8 +63,9 @@ constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TBN
 enum { T_QKV = 0, T_RESID = 1, T_SWIGLU = 2 };
 
 struct TcParams {
-    int M, N, K;  // N: output columns (QKV, RESID) or F (SWIGLU)
-    int n_tiles;  // output tiles along N
+    int M, N, K;      // N: output columns (QKV, RESID) or F (SWIGLU)
+    int tile0, tile1;  // output tiles of this launch (of m_tiles * n_tiles, M fastest)
+    int ksplit;        // CTAs (one cluster) that share a tile's K, 1 without clusters
     float* x;
     uint16_t* a;  // SWIGLU output: split pair [2][M][N] (hi plane, then lo plane)
     float* q;
@@ -133,20 +136,6 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
     d |= (uint64_t)1 << 46;              // descriptor version
     d |= (uint64_t)2 << 61;              // 128-byte swizzle
     return d;
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%"
-        "19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
@@ -301,6 +290,32 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// Every thread of the cluster; a hardware barrier that each of them reaches on
+// every path, also after an abort.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void st_cluster4(uint32_t addr, uint32_t rank, float a, float b, float c, float d) {
+    asm volatile(
+        "{\n .reg .b32 r;\n mapa.shared::cluster.u32 r, %0, %1;\n st.shared::cluster.v4.f32 [r], {%2,%3,%4,%5};\n}\n" ::"r"(
+            addr),
+        "r"(rank), "f"(a), "f"(b), "f"(c), "f"(d)
+        : "memory");
+}
+
+template <int EPI>
+__device__ __forceinline__ void epilogue(const TcParams& p, float (&acc)[128], int row, int ntile, int h) {
+    if (EPI == T_RESID) {
+        epi_resid(p, acc, row, ntile * TBN + 128 * h);
+    } else if (EPI == T_SWIGLU) {
+        epi_swiglu(p, acc, row, ntile * 128 + 64 * h);
+    } else if (p.d == 128) {
+        epi_qkv<128>(p, acc, row, ntile * TBN + 128 * h);
+    } else {
+        epi_qkv<64>(p, acc, row, ntile * TBN + 128 * h);
+    }
+}
+
 // Persistent tensor-core GEMM.  CTA b takes output tiles b, b + grid, ... in
 // M-fastest order (the CTAs sharing a weight tile run together, so it is read
 // from HBM about once).  Roles:
@@ -317,6 +332,14 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // number of MMAs summed into one accumulator, biased toward zero); summing at
 // most KC k-blocks there and the chunks in fp32 keeps the product at fp32-GEMV
 // accuracy.
+//
+// CL: a launch with fewer tiles than SMs (short prompts, row-poor matrices, or
+// the tiles past the last full wave).  A cluster of ksplit CTAs shares one tile:
+// CTA r takes the r-th part of K, and once every CTA has drained its last chunk
+// the partial sums meet through distributed shared memory, in the ring's space
+// (idle by then, since such a cluster has one tile only): each CTA owns a range
+// of the tile's rows, receives the others' sums for them, adds them in rank
+// order (the result does not depend on scheduling) and runs the epilogue.
 constexpr int kEpiWarps = 8;
 constexpr int kThreadsTC = 64 + 32 * kEpiWarps;
 constexpr uint32_t kTmemCols = 512;
@@ -325,7 +348,7 @@ constexpr int KC = 16;  // k-blocks per accumulation chunk (K = 1024)
 // 10 warps: the SM's four register partitions (16K each) hold three warps in
 // two of them, so at most 168 registers per thread -- enough for an epilogue
 // thread's 128 fp32 running sums (a few words spill around the epilogue)
-template <int EPI, int SPLIT>
+template <int EPI, int SPLIT, bool CL>
 __global__ void __launch_bounds__(kThreadsTC, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAlo,
                    const __grid_constant__ CUtensorMap tmB0, const __grid_constant__ CUtensorMap tmB1, TcParams p) {
@@ -338,9 +361,11 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m_tiles = (p.M + TBM - 1) / TBM;
-    const int n_total = m_tiles * p.n_tiles;
     const int nk = (p.K + TBK - 1) / TBK;
-    const int nchunks = (nk + KC - 1) / KC;
+    const int rank = CL ? (int)(blockIdx.x % p.ksplit) : 0;
+    const int kb_lo = CL ? nk * rank / p.ksplit : 0, kb_hi = CL ? nk * (rank + 1) / p.ksplit : nk;
+    const int nchunks = (kb_hi - kb_lo + KC - 1) / KC;
+    const int t_first = p.tile0 + (CL ? blockIdx.x / p.ksplit : blockIdx.x), t_step = CL ? p.tile1 : gridDim.x;
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES);
     const uint32_t cfull0 = smem_u32(bars + 2 * STAGES), cempty0 = smem_u32(bars + 2 * STAGES + 2);
     const uint32_t done_bar = smem_u32(bars + 2 * STAGES + 4);
@@ -373,11 +398,11 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
         if (lane == 0) {
             const CUtensorMap* mb1 = (EPI == T_SWIGLU) ? &tmB1 : &tmB0;
             int kbg = 0;  // k-blocks issued by this CTA, over all its tiles
-            for (int t = blockIdx.x; t < n_total && !*abort; t += gridDim.x) {
+            for (int t = t_first; t < p.tile1 && !*abort; t += t_step) {
                 const int m0 = (t % m_tiles) * TBM, ntile = t / m_tiles;
                 const int y0 = (EPI == T_SWIGLU) ? ntile * 128 : ntile * TBN;
                 const int y1 = (EPI == T_SWIGLU) ? ntile * 128 : ntile * TBN + 128;
-                for (int kb = 0; kb < nk; ++kb, ++kbg) {
+                for (int kb = kb_lo; kb < kb_hi; ++kb, ++kbg) {
                     const int s = kbg % STAGES;
                     if (!mbar_wait_ab(empty0 + 8 * s, ((kbg / STAGES) & 1) ^ 1, abort)) {
                         record_error(1);
@@ -401,7 +426,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
         if (lane == 0) {
             int kbg = 0, cg = 0;  // k-blocks and chunks consumed by this CTA
             bool ok = true;
-            for (int t = blockIdx.x; t < n_total && ok; t += gridDim.x) {
+            for (int t = t_first; t < p.tile1 && ok; t += t_step) {
                 for (int c = 0; c < nchunks && ok; ++c, ++cg) {
                     const int b = cg & 1;
                     if (!mbar_wait_ab(cempty0 + 8 * b, ((cg >> 1) & 1) ^ 1, abort)) {  // drained by the epilogue
@@ -411,8 +436,8 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t acc = tmem + (uint32_t)(b * TBN);
-                    const int kb1 = (c + 1) * KC < nk ? (c + 1) * KC : nk;
-                    for (int kb = c * KC; kb < kb1; ++kb, ++kbg) {
+                    const int kb0 = kb_lo + c * KC, kb1 = kb0 + KC < kb_hi ? kb0 + KC : kb_hi;
+                    for (int kb = kb0; kb < kb1; ++kb, ++kbg) {
                         const int s = kbg % STAGES;
                         if (!mbar_wait_ab(full0 + 8 * s, (kbg / STAGES) & 1, abort)) {
                             record_error(2);
@@ -424,7 +449,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
                         const uint64_t da = smem_desc(sa), db = smem_desc(sa + B_OFF);
 #pragma unroll
                         for (int k = 0; k < TBK / 16; ++k) {  // 32 bytes along K per instruction
-                            umma_bf16(acc, da + 2 * k, db + 2 * k, (kb != c * KC || k != 0) ? 1u : 0u);
+                            umma_bf16(acc, da + 2 * k, db + 2 * k, (kb != kb0 || k != 0) ? 1u : 0u);
                             if (SPLIT) umma_bf16(acc, smem_desc(sa + A_BYTES) + 2 * k, db + 2 * k, 1u);  // + A_lo W^T
                         }
                         umma_commit(empty0 + 8 * s);
@@ -441,7 +466,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
         const int q = warp & 3, h = (warp - 2) >> 2;  // TMEM lane quadrant, column half
         int cg = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < n_total && ok; t += gridDim.x) {
+        for (int t = t_first; t < p.tile1 && ok; t += t_step) {
             const int m0 = (t % m_tiles) * TBM, ntile = t / m_tiles;
             const int row = m0 + q * 32 + lane;
             float acc[128];
@@ -467,18 +492,49 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(cempty0 + 8 * b);
             }
-            if (!ok || row >= p.M) continue;
-            if (EPI == T_RESID) {
-                epi_resid(p, acc, row, ntile * TBN + 128 * h);
-            } else if (EPI == T_SWIGLU) {
-                epi_swiglu(p, acc, row, ntile * 128 + 64 * h);
-            } else {
-                if (p.d == 128)
-                    epi_qkv<128>(p, acc, row, ntile * TBN + 128 * h);
-                else
-                    epi_qkv<64>(p, acc, row, ntile * TBN + 128 * h);
+            if constexpr (CL) {
+                // sums to the CTAs that own their rows: [source][column / 4][row], 16
+                // bytes each, so that a warp's rows are contiguous
+                const int rows = p.M - m0 < TBM ? p.M - m0 : TBM;
+                const int per = (rows + p.ksplit - 1) / p.ksplit;
+                const int tr = q * 32 + lane, owner = tr / per, lr = tr - owner * per;
+                const uint32_t buf = smem_u32(smem);
+                __syncwarp();
+                cluster_sync();
+                if (tr < rows && owner != rank) {
+                    const uint32_t at = buf + (uint32_t)(((rank * 64 + h * 32) * per + lr) * 16);
+#pragma unroll
+                    for (int j = 0; j < 128; j += 4)
+                        st_cluster4(at + (uint32_t)((j / 4) * per * 16), (uint32_t)owner, acc[j], acc[j + 1], acc[j + 2],
+                                    acc[j + 3]);
+                }
+                __syncwarp();
+                cluster_sync();
+                if (tr < rows && owner == rank && ok) {
+                    for (int src = 0; src < p.ksplit; ++src) {
+                        if (src == rank) continue;
+                        const float4* in =
+                            reinterpret_cast<const float4*>(smem) + (size_t)(src * 64 + h * 32) * per + lr;
+#pragma unroll
+                        for (int j = 0; j < 128; j += 4) {
+                            const float4 v = in[(j / 4) * per];
+                            acc[j] += v.x;
+                            acc[j + 1] += v.y;
+                            acc[j + 2] += v.z;
+                            acc[j + 3] += v.w;
+                        }
+                    }
+                    epilogue<EPI>(p, acc, row, ntile, h);
+                }
+                ok = false;  // one tile per cluster
+            } else if (ok && row < p.M) {
+                epilogue<EPI>(p, acc, row, ntile, h);
             }
         }
+    }
+    if (CL && warp < 2) {  // the exchange's two barriers
+        cluster_sync();
+        cluster_sync();
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -513,39 +569,90 @@ cudaError_t make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t K)
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+template <int EPI, int SPLIT, bool CL>
+cudaError_t launch_grid(const CUtensorMap (&m)[4], const TcParams& p, int ctas, cudaStream_t st, int* max_clusters) {
+    constexpr int SMEM = Ring<SPLIT>::SMEM_BYTES;
+    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<EPI, SPLIT, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         SMEM);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(kThreadsTC);
+    cfg.dynamicSmemBytes = SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = p.ksplit;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = CL ? at : nullptr;
+    cfg.numAttrs = CL ? 1 : 0;
+    if (max_clusters) return cudaOccupancyMaxActiveClusters(max_clusters, tc_gemm_kernel<EPI, SPLIT, CL>, &cfg);
+    return cudaLaunchKernelEx(&cfg, tc_gemm_kernel<EPI, SPLIT, CL>, m[0], m[1], m[2], m[3], p);
+}
+
+// CTAs per tile for a launch of `tiles` tiles: the split whose longest CTA takes
+// the fewest k-blocks, every cluster resident at once.  The exchange costs about
+// as much as kExchange k-blocks (4 us), and so does the start of a second launch
+// (`more` tiles before these).  A cluster lies inside one GPC, so how
+// many fit is asked of the device, once per size.
+constexpr int kMaxSplit = 8, kExchange = 6;
+template <int EPI, int SPLIT>
+cudaError_t choose_split(const CUtensorMap (&m)[4], TcParams p, int tiles, bool more, int nk, int dev, int* out) {
+    static std::atomic<int> fit[64][kMaxSplit + 1];  // clusters of each size that fit a device at once (0: not asked)
+    *out = 1;
+    int best = nk;
+    for (int s = 2; s <= kMaxSplit && s * 4 <= nk; ++s) {
+        int n = dev < 64 ? fit[dev][s].load(std::memory_order_relaxed) : 0;
+        if (n == 0) {
+            p.ksplit = s;
+            const cudaError_t e = launch_grid<EPI, SPLIT, true>(m, p, s, nullptr, &n);
+            if (e != cudaSuccess) return e;
+            if (dev < 64) fit[dev][s].store(n, std::memory_order_relaxed);
+        }
+        const int cost = (nk + s - 1) / s + kExchange + (more ? kExchange : 0);
+        if (tiles <= n && cost < best) {
+            best = cost;
+            *out = s;
+        }
+    }
+    return cudaSuccess;
+}
+
 template <int EPI, int SPLIT>
 cudaError_t launch_tc_t(const void* A, const void* W0, const void* W1, uint64_t w_rows, TcParams& p, int n_tiles,
                         cudaStream_t st) {
     cudaError_t e = encoder();
     if (e != cudaSuccess) return e;
     if (p.M <= 0 || n_tiles <= 0) return cudaSuccess;
-    CUtensorMap ma, malo, mb0, mb1;
+    CUtensorMap m[4];
     const uint16_t* A16 = static_cast<const uint16_t*>(A);
-    if ((e = make_map(&ma, A16, (uint64_t)p.M, (uint64_t)p.K)) != cudaSuccess) return e;
+    if ((e = make_map(&m[0], A16, (uint64_t)p.M, (uint64_t)p.K)) != cudaSuccess) return e;
     // the lo plane follows the hi plane (M * K elements on)
-    if ((e = make_map(&malo, SPLIT ? A16 + (size_t)p.M * p.K : A16, (uint64_t)p.M, (uint64_t)p.K)) != cudaSuccess)
+    if ((e = make_map(&m[1], SPLIT ? A16 + (size_t)p.M * p.K : A16, (uint64_t)p.M, (uint64_t)p.K)) != cudaSuccess)
         return e;
-    if ((e = make_map(&mb0, W0, w_rows, (uint64_t)p.K)) != cudaSuccess) return e;
-    if ((e = make_map(&mb1, W1 ? W1 : W0, w_rows, (uint64_t)p.K)) != cudaSuccess) return e;
-    constexpr int SMEM = Ring<SPLIT>::SMEM_BYTES;
-    static bool attr = false;
-    if (!attr) {
-        e = cudaFuncSetAttribute(tc_gemm_kernel<EPI, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    if ((e = make_map(&m[2], W0, w_rows, (uint64_t)p.K)) != cudaSuccess) return e;
+    if ((e = make_map(&m[3], W1 ? W1 : W0, w_rows, (uint64_t)p.K)) != cudaSuccess) return e;
+    int dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     // persistent: one CTA per SM (the ring takes most of the shared memory), at
-    // most one per tile
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    }
-    p.n_tiles = n_tiles;
-    const int tiles = ((p.M + TBM - 1) / TBM) * n_tiles;
-    tc_gemm_kernel<EPI, SPLIT><<<tiles < sms ? tiles : sms, kThreadsTC, SMEM, st>>>(ma, malo, mb0, mb1, p);
-    return cudaGetLastError();
+    // most one per tile.  The tiles past the last full wave go to a launch of
+    // their own that splits their K over clusters, where that pays.
+    const int tiles = ((p.M + TBM - 1) / TBM) * n_tiles, nk = (p.K + TBK - 1) / TBK;
+    const int rest = tiles % sms;
+    int s = 1;
+    if (rest && (e = choose_split<EPI, SPLIT>(m, p, rest, tiles > sms, nk, dev, &s)) != cudaSuccess) return e;
+    p.tile0 = 0;
+    p.tile1 = s > 1 ? tiles - rest : tiles;
+    p.ksplit = 1;
+    if (p.tile1 > 0 &&
+        (e = launch_grid<EPI, SPLIT, false>(m, p, p.tile1 < sms ? p.tile1 : sms, st, nullptr)) != cudaSuccess)
+        return e;
+    if (s == 1) return cudaSuccess;
+    p.tile0 = p.tile1;
+    p.tile1 = tiles;
+    p.ksplit = s;
+    return launch_grid<EPI, SPLIT, true>(m, p, rest * s, st, nullptr);
 }
 
 template <int EPI>

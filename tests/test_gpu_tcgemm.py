@@ -79,3 +79,29 @@ def test_tc_gemm_split_parity(orc, M, N, K, rows):
         # and far inside what one bf16 plane allows: the lo plane is really used
         worst = max(worst, float(np.max(np.abs(got[m] - want) / (np.abs(W64) @ np.abs(A[m] - hi[m]) + 1e-30))))
     assert worst < 0.25
+
+
+# launches with few tiles, or few past the last full wave of 152, share a tile's
+# K among a cluster: one and several tiles of rows, row ranges that do not divide
+# evenly, K that does not divide into whole parts, a last wave of 8 tiles
+@pytest.mark.parametrize("M,N,K", [(1, 4, 2048), (17, 5120, 2112), (129, 5120, 2056), (130, 1000, 13824),
+                                   (88, 15360, 5120), (2048, 2560, 1032)])
+def test_tc_gemm_shared_k(M, N, K):
+    torch = need_gpu()
+    from paper_2512_21835_gb300 import loip as L
+    gen = torch.Generator("cuda").manual_seed(M + N + K)
+    A = torch.randn(M, K, generator=gen, device="cuda")
+    hi = A.bfloat16()
+    A2 = torch.stack([hi, (A - hi.float()).bfloat16()])
+    W = (torch.randn(N, K, generator=gen, device="cuda") * 0.02).bfloat16()
+    x0 = torch.randn(M, N, generator=gen, device="cuda")
+    x, again = x0.clone(), x0.clone()
+    L.loip_k_gemm_split(A2, W, x)
+    L.loip_k_gemm_split(A2, W, again)
+    assert L.loip_k_tc_status() == 0
+    a, w = A2[0].double() + A2[1].double(), W.double()
+    want = x0.double() + a @ w.T
+    # the fp32 summation bound of the pair's 2 K products
+    tol = (2 * K + 16) * 2.0 ** -24 * (a.abs() @ w.abs().T) + 4 * 2.0 ** -24 * want.abs()
+    assert bool(((x.double() - want).abs() <= tol).all())
+    assert torch.equal(x, again)  # the parts are added in a fixed order
