@@ -340,6 +340,9 @@ __device__ __forceinline__ void epilogue(const TcParams& p, float (&acc)[128], i
 // (idle by then, since such a cluster has one tile only): each CTA owns a range
 // of the tile's rows, receives the others' sums for them, adds them in rank
 // order (the result does not depend on scheduling) and runs the epilogue.
+// 13B projections of 88 rows (one CTA a tile in brackets): down 42 us (143), O 25
+// (63); 8B of 512 rows: down 81 (149), O 34 (55); 70B of 2048 rows, three full
+// waves and a shared fourth: down 1031 (1146), O 334 (362).
 constexpr int kEpiWarps = 8;
 constexpr int kThreadsTC = 64 + 32 * kEpiWarps;
 constexpr uint32_t kTmemCols = 512;

@@ -184,11 +184,11 @@ cudaError_t launch_unpack2(const uint8_t* in0, uint64_t n0, uint16_t* out0, cons
 cudaError_t tc_error(int* code);
 // Causal prefill attention on the tensor cores (attn_tc.cu).  tiles[i] =
 // {first row, rows, request, position of the first row}: a run of at most
-// attention_tc_tile_positions(Hq, Hkv) = 128 / (Hq / Hkv) consecutive positions
+// attention_tc_tile_positions(M, Hq, Hkv) consecutive positions
 // of one request, rows of q (fp32 [M, Hq d]); each row attends over its
 // request's cached positions 0 .. its own.  o: split pair [2][M][Hq d].
 // d = 64 or 128, Hq / Hkv = 1, 2, 4 or 8, page_tokens = 64.
-int attention_tc_tile_positions(int Hq, int Hkv);
+int attention_tc_tile_positions(int rows, int Hq, int Hkv);
 cudaError_t launch_attention_tc(const float* q, KvView kv, const int4* tiles, int n_tiles, int M, int Hq, int Hkv,
                                 int d, uint16_t* o, cudaStream_t st);
 cudaError_t attention_tc_error(int* code);

@@ -2233,7 +2233,6 @@ extern "C" int loip_prefill(loip_ctx* c, const int32_t* tokens, const int32_t* p
     rc = c->upload_page_table(s);
     if (rc) return rc;
     const int Mp = c->cfg.max_prefill_tokens;
-    const int tile_pos = attention_tc_tile_positions(c->Hq, c->Hkv);  // positions per attention tile
     // per-token request and position
     std::vector<int32_t> req_of(M), pos_of(M);
     std::vector<int32_t> last_row(n_prompts);
@@ -2257,7 +2256,8 @@ extern "C" int loip_prefill(loip_ctx* c, const int32_t* tokens, const int32_t* p
         memcpy(h, tokens + c0, (size_t)Mc * 4);
         memcpy(h + Mc, pos_of.data() + c0, (size_t)Mc * 4);
         memcpy(h + 2 * Mc, req_of.data() + c0, (size_t)Mc * 4);
-        // attention query tiles: runs of at most P_T consecutive rows of one request
+        // attention query tiles: runs of at most tile_pos consecutive rows of one request
+        const int tile_pos = attention_tc_tile_positions(Mc, c->Hq, c->Hkv);
         int32_t* ht = h + 3 * Mc;
         c->prefill_tiles = 0;
         for (int i = 0; i < Mc;) {
@@ -2579,12 +2579,17 @@ extern "C" int loip_k_prefill_attention(const float* q, const void* kv_base, con
         return LOIP_ERR_INVALID;
     const int G = Hq / Hkv;
     if (G != 1 && G != 2 && G != 4 && G != 8) return LOIP_ERR_INVALID;
-    const int tp = attention_tc_tile_positions(Hq, Hkv);
+    int64_t rows = 0;
+    for (int i = 0; i < n_prompts; ++i) {
+        const int len = prompt_lens[i], p0 = first_pos ? first_pos[i] : 0;
+        if (len < 1 || p0 < 0 || (int64_t)p0 + len > (int64_t)max_pages * page_tokens) return LOIP_ERR_INVALID;
+        rows += len;
+    }
+    const int tp = attention_tc_tile_positions((int)std::min<int64_t>(rows, 1 << 30), Hq, Hkv);
     std::vector<int4> t;
     int M = 0;
     for (int i = 0; i < n_prompts; ++i) {
         const int len = prompt_lens[i], p0 = first_pos ? first_pos[i] : 0;
-        if (len < 1 || p0 < 0 || (int64_t)p0 + len > (int64_t)max_pages * page_tokens) return LOIP_ERR_INVALID;
         for (int j = 0; j < len; j += tp) t.push_back(make_int4(M + j, std::min(tp, len - j), i, p0 + j));
         M += len;
     }
