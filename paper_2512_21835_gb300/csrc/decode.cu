@@ -25,6 +25,14 @@ constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
 constexpr int kStageFloats = 16384;  // 64 KB of staged activations per block
 constexpr int kMaxChunks = 256;      // pages per request in split attention (16384 positions)
+// Wide split attention runs a block per page up to this many blocks (pages of the
+// longest context x kv heads x requests) and on the tensor cores above: a short
+// launch is bound by latency, which the page blocks have less of (8B heads, 9
+// pages, batch 1: 10.8 us against 13.0), a long one by fp32 FMAs (70B heads, 512
+// pages: 22.9 against 20.9 us; 8192: 188 against 65). With fewer than four query
+// heads per kv head the page blocks hold out longer (40 heads, 1280 pages: 18.6
+// both).
+constexpr int kPageBlocks = 512, kPageBlocksFewHeads = 1280;
 #ifndef LOIP_GEMV_MIN_BLOCKS1
 #define LOIP_GEMV_MIN_BLOCKS1 2  // resident blocks per SM the registers are sized for
 #endif
@@ -1899,6 +1907,13 @@ cudaError_t launch_attention(const float* q, KvView kv, const int32_t* ctx_lens,
     p.Hkv = Hkv;
     p.max_chunks = (max_ctx + kv.page_tokens - 1) / kv.page_tokens;
     if (split && p.max_chunks > kMaxChunks) return cudaErrorInvalidValue;
+    const int64_t blocks = (int64_t)p.max_chunks * Hkv * B;
+    if (split && wide && !o_split && blocks >= (Hq >= 4 * Hkv ? kPageBlocks : kPageBlocksFewHeads)) {
+        return launch_attention_decode(q, kv, ctx_lens, positions, row_req, B, Hq, Hkv, d, p.max_chunks, scratch,
+                                       attention_counters(scratch, scratch_rows < B ? B : scratch_rows, Hq, d, max_ctx,
+                                                          kv.page_tokens),
+                                       static_cast<float*>(o), st, pdl);
+    }
     p.scale = 1.0f / sqrtf((float)d);
     p.scratch = scratch;
     if (scratch_rows < B) scratch_rows = B;

@@ -1,6 +1,7 @@
-"""Prefill attention where its tiling can go wrong (tiles of one and of two
-128-row halves, halves that end on different pages or hold a single row), against
-the fp64 softmax within the error of the split operands."""
+"""Attention where its tiling can go wrong, against the fp64 softmax: prefill (tiles
+of one and of two 128-row halves, halves that end on different pages or hold a
+single row) within the error of the split operands; decode on the tensor cores
+(one and several pages a block, one block and many a request) at fp32."""
 import math
 
 import numpy as np
@@ -76,3 +77,60 @@ def test_prefill_halves(L, Hq, Hkv, d, lens, first):
         tol = 2.0 ** -17 * (8 * math.sqrt(d) + 4) * mag + 1e-6
         assert bool(((got[at:at + n] - want).abs() <= tol).all())
         at += n
+
+
+# max_ctx decides for the tensor cores (512 pages over all requests and kv heads,
+# 1280 with fewer than four query heads each); the lengths for the pages per block
+@pytest.mark.parametrize("Hq,Hkv,d,max_ctx,lens", [
+    (64, 8, 128, 4096, (1,)), (64, 8, 128, 4096, (4096,)), (32, 8, 128, 16384, (16384, 17, 4033, 64)),
+    (40, 40, 128, 4096, (65, 2111)), (16, 8, 64, 8192, (15, 16, 8191)), (8, 8, 64, 16384, (16321,)),
+    (64, 8, 128, 1088, (1088, 63, 1, 640, 129, 1025, 48, 700))])
+def test_decode_long(L, Hq, Hkv, d, max_ctx, lens):
+    import torch
+    kv, table, page_bytes, flat = paged(lens, Hkv, d, 5)
+    B, pages = len(lens), max_ctx // P
+    assert pages * Hkv * B >= (512 if Hq >= 4 * Hkv else 1280)
+    pt = torch.zeros(B, pages, dtype=torch.int64, device="cuda")
+    pt[:, :table.shape[1]] = table
+    q = torch.randn(B, Hq * d, generator=torch.Generator("cuda").manual_seed(6), device="cuda")
+    scratch = torch.empty(L.loip_k_attention_scratch_floats(B, Hq, d, max_ctx, P), device="cuda")
+    o, again = torch.empty(B, Hq * d, device="cuda"), torch.empty(B, Hq * d, device="cuda")
+    ctx = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    for out in (o, again):
+        L.loip_k_attention(q, kv, pt, pages, ctx, Hq, Hkv, d, P, 0, page_bytes, max_ctx, scratch, out)
+    assert torch.equal(o, again)
+    for b, n in enumerate(lens):
+        want, mag = softmax_rows(q[b:b + 1].double().view(1, Hq, d), *flat[b],
+                                 torch.tensor([n - 1], device="cuda"))
+        # scores: d-term fp32 sums of |q||k|/sqrt d ~ sqrt d, which scale the weights;
+        # outputs: up to n/16 weighted adds per warp
+        tol = 2.0 ** -24 * ((d + 16) * 4 + n / 16 + 64) * mag + 1e-9
+        assert bool(((o[b].double().view(1, Hq, d) - want).abs() <= tol).all())
+
+
+def test_decode_infinities(L):
+    """As in plain fp32: an infinite value reaches the outputs of its dim only, an
+    infinitely low score has weight zero, an infinitely high one gives NaN."""
+    import torch
+    Hq, Hkv, d, n, max_ctx = 8, 1, 128, 700, 16384
+    page_bytes, pages, B = 2 * Hkv * P * d * 2, max_ctx // P, 2
+    kv = torch.randn(11, 2, Hkv, P, d, generator=torch.Generator("cuda").manual_seed(7), device="cuda").to(torch.bfloat16)
+    pt = torch.zeros(B, pages, dtype=torch.int64, device="cuda")
+    pt[:, :11] = torch.arange(11, device="cuda") * page_bytes
+    q = torch.randn(B, Hq * d, device="cuda").abs()
+    q[1].neg_()  # request 1 scores the infinite key infinitely high
+    kv[3, 1, 0, 20, 5] = float("inf")
+    kv[6, 0, 0, 33, 9] = float("-inf")
+    assert pages * Hkv * B >= 512
+    scratch = torch.empty(L.loip_k_attention_scratch_floats(B, Hq, d, max_ctx, P), device="cuda")
+    o = torch.empty(B, Hq * d, device="cuda")
+    L.loip_k_attention(q, kv, pt, pages, torch.tensor([n, n], dtype=torch.int32, device="cuda"), Hq, Hkv, d, P, 0,
+                       page_bytes, max_ctx, scratch, o)
+    o = o.view(B, Hq, d)
+    assert bool(torch.isinf(o[0, :, 5]).all()) and bool((o[0, :, 5] > 0).all())
+    fine = torch.ones(d, dtype=torch.bool, device="cuda")
+    fine[5] = False
+    k, v = (kv[:, i].permute(0, 2, 1, 3).reshape(-1, d)[:n].double() for i in (0, 1))
+    w = torch.softmax(q[0].double().view(Hq, d) @ k.T / math.sqrt(d), -1)
+    assert torch.allclose(o[0][:, fine].double(), (w @ v)[:, fine], rtol=1e-4, atol=1e-5)
+    assert bool(torch.isnan(o[1]).all())
