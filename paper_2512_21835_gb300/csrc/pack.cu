@@ -215,7 +215,19 @@ struct UnpackSeg {
     uint32_t blocks;
 };
 
-__global__ void __launch_bounds__(256) unpack_kernel(UnpackSeg s0, UnpackSeg s1) {
+// The decoder is bound by the ALU pipe (shifts, logic, permutes) while the FMA
+// pipe, which multiplies integers, idles.  So a field f of a word v moves up by n
+// bits as v + (2^n - 1) f; the factors are kernel arguments, or the compiler would
+// turn the multiplications back into shifts.  65536 superblocks (94 MB read, 134 MB
+// written): 59.4 us with shifts and a scan per quarter, 53.3 to 55.3 now; the ALU pipe
+// is busy 76 % of the time (before 92 %), 667 instructions per superblock and warp.
+struct UnpackMul {
+    uint32_t x255, x15, x3;  // moves by 8, 4 and 2 bits
+    uint32_t x128;           // << 7
+    uint32_t neg;            // -1
+};
+
+__global__ void __launch_bounds__(256) unpack_kernel(UnpackSeg s0, UnpackSeg s1, UnpackMul mul) {
     const bool second = blockIdx.x >= s0.blocks;
     const uint8_t* __restrict__ in = second ? s1.in : s0.in;
     uint16_t* __restrict__ out = second ? s1.out : s0.out;
@@ -238,100 +250,105 @@ __global__ void __launch_bounds__(256) unpack_kernel(UnpackSeg s0, UnpackSeg s1)
     const uint32_t emax = r0 & 0xffu;
     const uint64_t ranks = (uint64_t)(r0 >> 16) | ((uint64_t)__shfl_sync(0xffffffffu, r, 1) << 16);
     const uint32_t n_exc = __shfl_sync(0xffffffffu, r, 2) >> 24;
-    // level-1 escapes per quarter (c = 3: both bits set), and each lane's first:
+    // 2-bit fields at bits 2j -> 4-bit fields at bits 4j (j < 8)
+    auto spread2 = [&](uint32_t v) -> uint32_t {
+        v += (v & 0xff00u) * mul.x255;
+        v += (v & 0x00f000f0u) * mul.x15;
+        return v + (v & 0x0c0c0c0cu) * mul.x3;
+    };
+    // every byte to 0xff or 0 by its top bit
+    auto byte_sign = [](uint32_t v) -> uint32_t {
+        uint32_t m;
+        asm("prmt.b32 %0, %1, %1, 0xba98;" : "=r"(m) : "r"(v));
+        return m;
+    };
+    // first of this lane's entries of a level, by quarter, from the lane's counts:
     // two quarters' counts per scan, in 16-bit halves (at most 256 per quarter)
-    uint32_t n1[4], off1[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) n1[q] = __popc(c16[q] & (c16[q] >> 1) & 0x5555u);
-    {
+    auto offsets = [&](const uint32_t (&n)[4], uint32_t (&off)[4]) {
         uint32_t ta, tb;
-        const uint32_t xa = warp_excl_scan(n1[0] | (n1[1] << 16), lane, &ta);
-        const uint32_t xb = warp_excl_scan(n1[2] | (n1[3] << 16), lane, &tb);
-        const uint32_t t0 = ta & 0xffffu, t1 = ta >> 16, t2 = tb & 0xffffu;
-        off1[0] = xa & 0xffffu;
-        off1[1] = t0 + (xa >> 16);
-        off1[2] = t0 + t1 + (xb & 0xffffu);
-        off1[3] = t0 + t1 + t2 + (xb >> 16);
-    }
-    // this lane's level-2 codes (at most 8 per quarter: 16 bits of a 2-word window)
-    uint32_t l2[4], n2[4], off2[4];
+        const uint32_t xa = warp_excl_scan(n[0] + (n[1] << 16), lane, &ta);
+        const uint32_t xb = warp_excl_scan(n[2] + (n[3] << 16), lane, &tb);
+        const uint32_t t0 = ta & 0xffffu, t01 = t0 + (ta >> 16), t2 = tb & 0xffffu;
+        off[0] = xa & 0xffffu;
+        off[1] = t0 + (xa >> 16);
+        off[2] = t01 + (xb & 0xffffu);
+        off[3] = t01 + t2 + (xb >> 16);
+    };
+    // level-1 codes as nibbles (word e: nibble e) and the escapes (c = 3) among them
+    uint32_t sel[4], esc[4], n1[4], off1[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const uint32_t wi = off1[q] >> 4, sh = 2 * (off1[q] & 15);
-        const uint32_t lo = __shfl_sync(0xffffffffu, lv, (int)wi & 31);
-        const uint32_t hi = __shfl_sync(0xffffffffu, lv, (int)(wi + 1) & 31);
-        l2[q] = __funnelshift_r(lo, hi, sh) & (n1[q] ? 0xffffu >> (16 - 2 * n1[q]) : 0u);
-        n2[q] = __popc(l2[q] & (l2[q] >> 1) & 0x5555u);
+        sel[q] = spread2(c16[q]);
+        esc[q] = sel[q] & (sel[q] >> 1) & 0x11111111u;
+        n1[q] = __popc(esc[q]);
     }
-    {
-        uint32_t ta, tb;
-        const uint32_t xa = warp_excl_scan(n2[0] | (n2[1] << 16), lane, &ta);
-        const uint32_t xb = warp_excl_scan(n2[2] | (n2[3] << 16), lane, &tb);
-        const uint32_t t0 = ta & 0xffffu, t1 = ta >> 16, t2 = tb & 0xffffu;
-        off2[0] = xa & 0xffffu;
-        off2[1] = t0 + (xa >> 16);
-        off2[2] = t0 + t1 + (xb & 0xffffu);
-        off2[3] = t0 + t1 + t2 + (xb >> 16);
-    }
+    offsets(n1, off1);
     // k of four words at once: the level-1 codes select bytes of the first three
     // ranks; code 3 selects 0xff, which marks the escapes (no k is above 14)
     const uint32_t R1 = (uint32_t)(ranks & 0xffffffu) | 0xff000000u;
     const uint32_t R2 = (uint32_t)((ranks >> 24) & 0xffffffu) | 0xff000000u;  // ranks 3..5, 0xff: level 3
-    const uint32_t E4 = emax * 0x01010101u;
-    // 2-bit fields at bits 2j -> 4-bit fields at bits 4j (j < 8)
-    auto spread2 = [](uint32_t v) -> uint32_t {
-        v = (v | (v << 8)) & 0x00ff00ffu;
-        v = (v | (v << 4)) & 0x0f0f0f0fu;
-        return (v | (v << 2)) & 0x33333333u;
-    };
-    uint4 o[4];
+    uint32_t k03[4], k47[4], n2[4], off2[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const uint32_t sel = spread2(c16[q]);  // nibble e = level-1 code of word e
-        uint32_t k03 = __byte_perm(R1, 0u, sel), k47 = __byte_perm(R1, 0u, sel >> 16);
+        // this lane's level-2 codes (at most 8 per quarter: 16 bits of a 2-word
+        // window; what follows them in the window is never selected)
+        const uint32_t wi = off1[q] >> 4;
+        const uint32_t lo = __shfl_sync(0xffffffffu, lv, (int)wi & 31);
+        const uint32_t hi = __shfl_sync(0xffffffffu, lv, (int)(wi + 1) & 31);
+        const uint32_t l2 = __funnelshift_r(lo, hi, 2 * off1[q]) & 0xffffu;
+        k03[q] = __byte_perm(R1, 0u, sel[q]);
+        k47[q] = __byte_perm(R1, 0u, sel[q] >> 16);
         // level 2 without a loop: T holds, for the lane's j-th escape of the
         // quarter, the k its level-2 code names (0xff: level 3); escape word e
         // takes entry rank(e), the number of escapes before it (a nibble-wise
         // prefix product)
-        const uint32_t escN = sel & (sel >> 1) & 0x11111111u;  // nibble e = 1: word e escapes
-        const uint32_t rk = escN * 0x11111111u - escN;
-        const uint32_t t4 = spread2(l2[q]);  // nibble j = the j-th level-2 code
+        const uint32_t rk = esc[q] * 0x11111110u;  // at most 7 in a nibble
+        const uint32_t t4 = spread2(l2);           // nibble j = the j-th level-2 code
         const uint32_t T0 = __byte_perm(R2, 0u, t4), T1 = __byte_perm(R2, 0u, t4 >> 16);
-        const uint32_t M03 = ((k03 & 0x80808080u) >> 7) * 0xffu, M47 = ((k47 & 0x80808080u) >> 7) * 0xffu;
-        k03 = (k03 & ~M03) | (__byte_perm(T0, T1, rk & 0x7777u) & M03);
-        k47 = (k47 & ~M47) | (__byte_perm(T0, T1, (rk >> 16) & 0x7777u) & M47);
+        const uint32_t M03 = byte_sign(k03[q]), M47 = byte_sign(k47[q]);
+        k03[q] = (k03[q] & ~M03) | (__byte_perm(T0, T1, rk) & M03);
+        k47[q] = (k47[q] & ~M47) | (__byte_perm(T0, T1, rk >> 16) & M47);
+        n2[q] = __popc(k03[q] & 0x80808080u) + __popc(k47[q] & 0x80808080u);
+    }
+    offsets(n2, off2);
+    const uint32_t E4 = emax * 0x01010101u;
+    uint4 o[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
         // level 3 (rare): the words still marked 0xff, in word order; this lane's
         // nibbles of the quarter (at most 8: a 2-word window of words 22..31,
         // shuffled by the whole warp)
-        const uint32_t wi = 22 + (off2[q] >> 3), sh = 4 * (off2[q] & 7);
+        const uint32_t wi = 22 + (off2[q] >> 3);
         const uint32_t lo = __shfl_sync(0xffffffffu, lv, (int)wi & 31);
         const uint32_t hi = __shfl_sync(0xffffffffu, lv, (int)(wi + 1) & 31);
-        uint32_t m03 = k03 & 0x80808080u, m47 = k47 & 0x80808080u;
-        if (m03 | m47) {
-            uint32_t l3 = wi < 32 ? __funnelshift_r(lo, wi + 1 < 32 ? hi : 0u, sh) : 0u;
+        if (n2[q]) {
+            uint32_t l3 = __funnelshift_r(lo, hi, 4 * off2[q]);  // (past word 31 there are no entries)
+            uint32_t m03 = k03[q] & 0x80808080u, m47 = k47[q] & 0x80808080u;
             while (m03) {
                 const uint32_t shb = (uint32_t)(__ffs(m03) - 8);  // 8 * byte
                 m03 &= m03 - 1;
-                k03 = (k03 & ~(0xffu << shb)) | ((l3 & 15u) << shb);  // 15: an exception, patched below
+                k03[q] = (k03[q] & ~(0xffu << shb)) | ((l3 & 15u) << shb);  // 15: an exception, patched below
                 l3 >>= 4;
             }
             while (m47) {
                 const uint32_t shb = (uint32_t)(__ffs(m47) - 8);
                 m47 &= m47 - 1;
-                k47 = (k47 & ~(0xffu << shb)) | ((l3 & 15u) << shb);
+                k47[q] = (k47[q] & ~(0xffu << shb)) | ((l3 & 15u) << shb);
                 l3 >>= 4;
             }
         }
         // exponent bytes: emax - k never borrows (k <= emax; the exception
-        // placeholder 15 only where emax >= 15)
-        const uint32_t x03 = E4 - k03, x47 = E4 - k47;
-        // two words per register: sign | exponent << 7 | mantissa
-        auto pair = [](uint32_t smb, uint32_t xb, uint32_t sel2) -> uint32_t {
-            const uint32_t t = __byte_perm(smb, 0u, sel2), ee = __byte_perm(xb, 0u, sel2);
-            return ((t & 0x00800080u) << 8) | (ee << 7) | (t & 0x007f007fu);
+        // placeholder 15 only where emax >= 15).  Then four words' high bytes (sign,
+        // exponent >> 1) and low bytes (exponent & 1, mantissa), interleaved.
+        auto words = [&](uint32_t smb, uint32_t k, uint32_t& w01, uint32_t& w23) {
+            const uint32_t x = k * mul.neg + E4;
+            const uint32_t high = (smb & 0x80808080u) | ((x >> 1) & 0x7f7f7f7fu);
+            const uint32_t low = (smb & 0x7f7f7f7fu) | ((x * mul.x128) & 0x80808080u);
+            w01 = __byte_perm(low, high, 0x5140);
+            w23 = __byte_perm(low, high, 0x7362);
         };
-        o[q] = make_uint4(pair(sm[q].x, x03, 0x4140u), pair(sm[q].x, x03, 0x4342u), pair(sm[q].y, x47, 0x4140u),
-                          pair(sm[q].y, x47, 0x4342u));
+        words(sm[q].x, k03[q], o[q].x, o[q].y);
+        words(sm[q].y, k47[q], o[q].z, o[q].w);
     }
     // exceptions, into the register of the lane that holds the word
     for (uint32_t m = 0; m < n_exc; ++m) {
@@ -375,7 +392,8 @@ cudaError_t launch_unpack2(const uint8_t* in0, uint64_t n0, uint16_t* out0, cons
         return cudaErrorInvalidValue;
     const UnpackSeg s0{in0, out0, n0, (uint32_t)((n0 + kWarps - 1) / kWarps)};
     const UnpackSeg s1{in1, out1, n1, (uint32_t)((n1 + kWarps - 1) / kWarps)};
-    unpack_kernel<<<s0.blocks + s1.blocks, 256, 0, st>>>(s0, s1);
+    const UnpackMul mul{255u, 15u, 3u, 128u, 0xffffffffu};
+    unpack_kernel<<<s0.blocks + s1.blocks, 256, 0, st>>>(s0, s1, mul);
     return cudaGetLastError();
 }
 
