@@ -2,14 +2,14 @@
 // sm_103a, plus the embedding gather, the LM head with greedy argmax and the
 // seeded weight generator.
 //
-// Every decode projection is a weight-stationary matrix-vector product that is
-// HBM bound: each bf16 weight byte is read exactly once with 128-bit streaming
-// loads (ld.global.nc.L1::no_allocate), the fp32 activation rows are staged in
-// shared memory in a bank-conflict-free permuted layout, each warp owns a few
-// output rows and reduces its partial sums with xor shuffles.  Normalisation,
-// rotary embedding, KV-cache append, SwiGLU, residual adds and the argmax are
-// fused into the prologue/epilogue of the product that produces their input,
-// so activations never take an extra trip through HBM.
+// A projection is a matrix-vector product bound by the weight stream: each bf16
+// weight byte is read exactly once.  Batches, and batch 1 with weights in device
+// memory, run in gemv_batch.cu; here are the batch-1 kernels for the LM head, small
+// matrices and weights in mapped host memory: 128-bit streaming loads
+// (ld.global.nc.L1::no_allocate) to registers, sums reduced by xor shuffles.
+// Normalisation, rotary embedding, KV-cache append, SwiGLU, residual adds and the
+// argmax are fused into the prologue/epilogue of the product that produces their
+// input, so activations never take an extra trip through HBM.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -215,8 +215,8 @@ __device__ __forceinline__ void unit_epilogue(const GemvParams& p, int unit, flo
     }
 }
 
-// Batch 1, row-rich matrices and weights in mapped host memory (gemv_batch.cu
-// serves larger batches).
+// Batch 1: the LM head, weights in mapped host memory, row-rich matrices whose rows
+// are no whole 64-column blocks.
 template <int EPI>
 __global__ void __launch_bounds__(kThreads, LOIP_GEMV_MIN_BLOCKS1) gemv_kernel(GemvParams p) {
     constexpr int U = UnitRows<EPI>::U;
@@ -594,9 +594,6 @@ __global__ void __launch_bounds__(kTileWarps * 32, 2) gemv_tile_kernel(GemvParam
     pdl_trigger();
     uint4 wa[kTileRows];
     tile_first_load<EPI>(p, blockIdx.x, wa);  // weights do not depend on the previous kernel
-    if (p.pf_stride > 0 && threadIdx.x < 32)
-        for (int t = blockIdx.x + p.pf_stride; t < (int)gridDim.x; t += p.pf_stride)
-            prefetch_tile<EPI>(p, t, threadIdx.x);
     pdl_wait();
     tile_gemv<EPI, false>(p, blockIdx.x, -1, wa, sm);
 }
@@ -620,19 +617,28 @@ __global__ void argmax_reduce_kernel(const uint64_t* keys, int nblocks, int BT, 
     if (threadIdx.x == 0 && b < B) tokens[b] = (int32_t)(0xffffffffu - (uint32_t)(s[0] & 0xffffffffu));
 }
 
+// Matrices below this many elements keep the tile kernel: there a launch is bound by
+// its host side and latency, and the ring's costs 0.5 us more (tensor maps; 8.3 us
+// against 7.8 back to back at 2048 x 2048 and below; 4096 x 2048 gate/up 10.4 against
+// 13.2).
+constexpr int64_t kRingMin = 1 << 22;
 template <int EPI>
 cudaError_t launch_gemv(GemvParams& p, cudaStream_t st, bool pdl, int* nblocks_out = nullptr) {
-    // Batch 1: matrices with few rows (QKV, O-proj, down) keep too few units per
-    // warp for the persistent kernel to ramp up; the block-tile kernel issues a
-    // whole tile at once.  Row-rich ones (gate/up, LM head) stream better
-    // persistent, and so does a QKV of more than 8192 rows (13B: 15360, two or
-    // more RoPE pairs per warp), whose tiles would take six waves.  Weights in
-    // mapped host memory always go to the persistent kernel: over the host link
-    // a tile's serial chunk loads along a long row (down, K = 28672) ran at
-    // 183 GB/s against the link's 211, which the persistent kernel reaches.
     if (p.B > 1) return launch_gemv_batch(EPI, p, st, pdl, nblocks_out);  // tensor cores: gemv_batch.cu
+    // Batch 1, weights in device memory, rows of whole 64-column blocks: the ring of
+    // bulk copies (8B step 2967 -> 2780 us, 70B layer 254 -> 239). The LM head
+    // streams at 6.9 TB/s through the persistent kernel and stays there.
+    if (EPI != EPI_LOGITS && !p.w_host && p.K % 64 == 0 && (int64_t)p.N * p.K > kRingMin)
+        return launch_gemv_ring(EPI, p, st, pdl);
+    // Otherwise: matrices with few rows keep too few units per warp for the
+    // persistent kernel to ramp up; the block-tile kernel issues a whole tile at
+    // once. Row-rich ones stream better persistent, and so does a QKV of more than
+    // 8192 rows (two or more RoPE pairs per warp), whose tiles would take six waves.
+    // Weights in mapped host memory always go to the persistent kernel: over the
+    // host link a tile's serial chunk loads along a long row (down, K = 28672) ran at
+    // 183 GB/s against the link's 211, which the persistent kernel reaches.
     const int rows = (EPI == EPI_SWIGLU) ? 2 * p.n_units : p.N;
-    if (p.B == 1 && !p.w_host && rows <= (EPI == EPI_QKV ? 8192 : 16384)) {
+    if (!p.w_host && rows <= (EPI == EPI_QKV ? 8192 : 16384)) {
         const int per_tile = (EPI == EPI_QKV || EPI == EPI_SWIGLU) ? kTileRows / 2 : kTileRows;
         const int units = (EPI == EPI_QKV || EPI == EPI_SWIGLU) ? p.n_units : p.N;
         const int tiles = (units + per_tile - 1) / per_tile;
@@ -1804,19 +1810,9 @@ cudaError_t launch_qkv_rope(const float* x, const uint16_t* g, const uint16_t* w
 }
 
 cudaError_t launch_resid_gemv(const float* in, const uint16_t* w, int B, int N, int K, float* x, cudaStream_t st,
-                              bool pdl, bool w_host, bool prefetch_waves) {
+                              bool pdl, bool w_host) {
     GemvParams p{};
     p.w_host = w_host;
-    if (prefetch_waves && !w_host) {  // two block-tile blocks are resident per SM
-        static int sms = 0;
-        if (!sms) {
-            int dev = 0;
-            if (cudaGetDevice(&dev) != cudaSuccess ||
-                cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-                sms = 0;
-        }
-        p.pf_stride = 2 * sms;
-    }
     p.in = in;
     p.w0 = w;
     p.B = B;

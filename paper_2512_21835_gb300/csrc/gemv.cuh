@@ -32,11 +32,10 @@ struct GemvParams {
     RopeFreqs rope;
     int w_host;  // weights are read in place from mapped host memory: no L2 prefetch of them
     float* qk_raw;  // QK-norm models: query/key rows leave unrotated here ([B][(Hq + 2 Hkv) d])
-    int pf_stride;  // block-tile kernel, > 0: before its dependency wait, block b pulls tiles
-                    // b + pf_stride, b + 2 pf_stride, ... (the later waves) into L2
 };
 
 cudaError_t launch_gemv_batch(int epi, const GemvParams& p, cudaStream_t st, bool pdl, int* nblocks_out);
+cudaError_t launch_gemv_ring(int epi, const GemvParams& p, cudaStream_t st, bool pdl);
 
 namespace {
 

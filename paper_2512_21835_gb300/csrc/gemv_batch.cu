@@ -1,5 +1,6 @@
-// gemv_batch.cu -- the decode projections for batches of 2 to 8 rows, on the
-// tensor cores (mma.sync m16n8k16).
+// gemv_batch.cu -- the decode projections on a ring of bulk copies: for batches of
+// 2 to 8 rows on the tensor cores (mma.sync m16n8k16), for batch 1 with fp32 FMAs
+// (further down).
 //
 // The product is bound by the weight stream, so the kernel is a deep ring of
 // bulk copies with just enough arithmetic behind it.  Eight fp32 activation
@@ -190,7 +191,6 @@ __global__ void __launch_bounds__(kBThreads, 1)
     const int n_chunks = (K + kBChunk - 1) / kBChunk;
     const int64_t step = half_step<EPI>(p);
 
-    pdl_trigger();
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(full0 + 8 * s, TMA ? 1 : 32);
@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(kBThreads, 1)
                         }
                     }
             }
+        pdl_trigger();
     done:
         if (*abort) {  // given up: the copies in flight land before the block's shared memory is released
             if (!TMA) asm volatile("cp.async.wait_all;" ::: "memory");
@@ -466,6 +467,252 @@ __global__ void __launch_bounds__(kBThreads, 1)
     }
 }
 
+// ----------------------------------------------------------------------------
+// Batch 1: the same ring and tiles, fp32 FMAs.  Eight consumer warps take one
+// 64-column block of a chunk each; a lane holds one 16-byte piece of it for four
+// rows of every tile, and the eight activations that meet it stay in registers
+// for all tiles of the chunk.  Eight products are summed from zero and then added
+// to the row's sum, so a chain of additions is K / 512 + 8 long.
+//
+// A step runs these kernels back to back, each bound by the weight stream, so
+// what is left to gain lies between them: the wait for the previous kernel, the
+// first activation loads and the last sums take about 2 us per launch, in which
+// nothing streams if the ring is already full.  So the next kernel is triggered
+// when a block has issued its last copy, and the ring takes most of the shared
+// memory: a block of the next launch then starts where one has ended, and fills
+// its ring during the gap.  8B step of 32 layers: 2967 -> 2780 us, 70B layer 254 ->
+// 239 (before: loads to registers, by blocks of eight rows for QKV, O and down and by
+// persistent warps for gate/up).  In one sweep: 2806 us; triggered at the start 2845;
+// with 6 stages, so that two launches share an SM and the ring fills long before the
+// gap, 3114 and 3470; with 16 more tiles copied ahead into L2 2804.
+// ----------------------------------------------------------------------------
+constexpr int kRW = 8;                   // consumer warps per block
+constexpr int kRThreads = kRW * 32 + 32;  // and the producer warp
+constexpr int kRT = 8;                   // tiles per pass
+constexpr int kRingSmem = 1024 + kStages * (int)kStageBytes;
+
+template <int EPI>
+__global__ void __launch_bounds__(kRThreads, 1)
+    gemv_ring_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
+                     const __grid_constant__ GemvParams p) {
+    constexpr int UPT = TileUnits<EPI>::U;
+    constexpr bool PAIRS = TileUnits<EPI>::PAIRS;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    __shared__ uint64_t s_full[kStages], s_empty[kStages];
+    __shared__ float s_red[kRW][kRT * 16];
+    __shared__ float s_ss[kRW];
+    __shared__ int s_abort;
+    volatile int* abort = &s_abort;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int K = p.K;
+    const uint32_t ring = smem_u32(smem), full0 = smem_u32(s_full), empty0 = smem_u32(s_empty);
+    const int all = (p.n_units + UPT - 1) / UPT;
+    const int tile0 = (int)((int64_t)all * blockIdx.x / gridDim.x);
+    const int n_tiles = (int)((int64_t)all * (blockIdx.x + 1) / gridDim.x) - tile0;
+    const int n_pass = (n_tiles + kRT - 1) / kRT;
+    const int tpp = (n_tiles + n_pass - 1) / n_pass;  // tiles per pass
+    const int n_chunks = (K + kBChunk - 1) / kBChunk;
+
+    if (tid == 0) {
+        for (int s = 0; s < kStages; ++s) {
+            mbar_init(full0 + 8 * s, 1);
+            mbar_init(empty0 + 8 * s, kRW);
+        }
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+
+    if (warp == kRW) {  // ---- producer: tiles in the order (pass, chunk, tile)
+        if (lane != 0) return;
+        int s = 0, n = 0;
+        uint32_t phase = 1;  // the first wait for each stage passes at once
+        for (int first = 0; first < n_tiles; first += tpp) {
+            const int nt = min(tpp, n_tiles - first);
+            for (int c = 0; c < n_chunks; ++c)
+                for (int t = 0; t < nt; ++t, ++n) {
+                    mbar_wait(empty0 + 8 * s, phase, abort);
+                    if (*abort) goto done;
+                    const int u0 = (tile0 + first + t) * UPT;
+                    const int row = unit_row0<EPI>(p, u0);
+                    const bool two = PAIRS || u0 + 8 < p.n_units;
+                    const uint32_t bar = full0 + 8 * s, dst = ring + (uint32_t)s * kStageBytes;
+                    mbar_expect_tx(bar, two ? kStageBytes : kGroupBytes);
+                    tma_load_3d(dst, &tm0, 0, row, c * (kBChunk / 64), bar);
+                    if (two)
+                        tma_load_3d(dst + kGroupBytes, EPI == EPI_SWIGLU ? &tm1 : &tm0, 0,
+                                    EPI == EPI_SWIGLU ? row : EPI == EPI_QKV ? row + (p.d >> 1) : row + 8,
+                                    c * (kBChunk / 64), bar);
+                    if (++s == kStages) {
+                        s = 0;
+                        phase ^= 1;
+                    }
+                }
+        }
+        pdl_trigger();
+    done:
+        if (*abort) {  // given up: the copies in flight land before the block's shared memory is released
+            int never = 0;
+            for (int k = max(0, n - kStages); k < n; ++k)
+                mbar_wait(full0 + 8 * (k % kStages), (k / kStages) & 1, &never);
+        }
+        return;
+    }
+
+    // ---- consumers: a lane holds eight columns (16-byte piece `piece` of the
+    // warp's 64) and takes rows r, r + 4, r + 8, r + 12 of every tile
+    const int piece = lane & 7, r = lane >> 3;
+    const bool norm = p.g != nullptr;
+    const int kw = warp * 64 + piece * 8;
+    uint32_t off[2];
+    off[0] = (uint32_t)(warp * 1024 + r * 128 + ((piece ^ r) << 4));
+    off[1] = (uint32_t)(warp * 1024 + (r + 4) * 128 + ((piece ^ (r + 4)) << 4));
+    pdl_wait();
+
+    float4 xa, xb;
+    uint4 gv;
+    auto load_x = [&](int c) {
+        const int k = c * kBChunk + kw;
+        xa = xb = make_float4(0.f, 0.f, 0.f, 0.f);
+        gv = make_uint4(0, 0, 0, 0);
+        if (k < K) {
+            xa = *reinterpret_cast<const float4*>(p.in + k);
+            xb = *reinterpret_cast<const float4*>(p.in + k + 4);
+            if (norm) gv = *reinterpret_cast<const uint4*>(p.g + k);
+        }
+    };
+    auto sync_consumers = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(kRW * 32) : "memory"); };
+    float ss = 0.f, inv = 1.f;
+    int s = 0;
+    uint32_t phase = 0;
+    load_x(0);
+    for (int first = 0; first < n_tiles; first += tpp) {
+        const int nt = min(tpp, n_tiles - first);
+        // what the epilogue needs from memory, early
+        const int n_out = nt * UPT, u = (tile0 + first) * UPT + tid;
+        const bool mine = tid < n_out && u < p.n_units;
+        float ea = 0.f, eb = 0.f;
+        int pos = 0, head = 0, j = 0;
+        if (EPI == EPI_RESID && mine) ea = p.out[u];
+        if (EPI == EPI_QKV && mine) {
+            pos = p.positions[0];
+            head = u / (p.d >> 1);
+            j = u - head * (p.d >> 1);
+            if (!p.qk_raw && head < p.Hq + p.Hkv) rope_cos_sin(pos, p.rope.inv_freq[j], &ea, &eb);
+        }
+        float acc[kRT][4];
+#pragma unroll
+        for (int t = 0; t < kRT; ++t) acc[t][0] = acc[t][1] = acc[t][2] = acc[t][3] = 0.f;
+#pragma unroll 1
+        for (int c = 0; c < n_chunks; ++c) {
+            float x[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+            if (norm) {
+                const float gf[8] = {bf_lo(gv.x), bf_hi(gv.x), bf_lo(gv.y), bf_hi(gv.y),
+                                     bf_lo(gv.z), bf_hi(gv.z), bf_lo(gv.w), bf_hi(gv.w)};
+                if (first == 0)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) ss = fmaf(x[e], x[e], ss);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) x[e] *= gf[e];
+            }
+            load_x(c + 1 < n_chunks ? c + 1 : 0);  // the next chunk's, or the next pass's first
+#pragma unroll
+            for (int t = 0; t < kRT; ++t) {
+                if (t >= nt) break;
+                mbar_wait(full0 + 8 * s, phase, abort);
+                const uint32_t src = ring + (uint32_t)s * kStageBytes;
+                uint4 w[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) w[i] = lds128(src + (i >> 1) * kGroupBytes + off[i & 1]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty0 + 8 * s);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float a = bf_lo(w[i].x) * x[0];
+                    a = fmaf(bf_hi(w[i].x), x[1], a);
+                    a = fmaf(bf_lo(w[i].y), x[2], a);
+                    a = fmaf(bf_hi(w[i].y), x[3], a);
+                    a = fmaf(bf_lo(w[i].z), x[4], a);
+                    a = fmaf(bf_hi(w[i].z), x[5], a);
+                    a = fmaf(bf_lo(w[i].w), x[6], a);
+                    a = fmaf(bf_hi(w[i].w), x[7], a);
+                    acc[t][i] += a;
+                }
+                if (++s == kStages) {
+                    s = 0;
+                    phase ^= 1;
+                }
+            }
+        }
+        // the eight lanes of a row, then the warps in order
+#pragma unroll
+        for (int t = 0; t < kRT; ++t) {
+            if (t >= nt) break;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float v = acc[t][i];
+#pragma unroll
+                for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (piece == 0) s_red[warp][t * 16 + r + 4 * i] = v;
+            }
+        }
+        if (first == 0 && norm) {
+            float q = ss;
+#pragma unroll
+            for (int o = 4; o; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+            if (lane == 0) s_ss[warp] = q;
+        }
+        sync_consumers();
+        if (first == 0 && norm) {
+            float q = 0.f;
+            for (int w = 0; w < kRW; ++w) q += s_ss[w];
+            inv = 1.0f / sqrtf(q / (float)K + p.eps);
+        }
+        if (mine && !*abort) {
+            const int slot = PAIRS ? (tid >> 3) * 16 + (tid & 7) : tid;
+            float v0 = 0.f, v1 = 0.f;
+#pragma unroll
+            for (int w = 0; w < kRW; ++w) {
+                v0 += s_red[w][slot];
+                if (PAIRS) v1 += s_red[w][slot + 8];
+            }
+            v0 *= inv;
+            v1 *= inv;
+            if (EPI == EPI_RESID) {
+                p.out[u] = ea + v0;
+            } else if (EPI == EPI_SWIGLU) {
+                p.out[u] = v0 / (1.0f + expf(-v0)) * v1;
+            } else {
+                const int hd = p.d >> 1;
+                if (p.qk_raw && head < p.Hq + p.Hkv) {  // normalised and rotated by qk_norm_rope_kernel
+                    p.qk_raw[(size_t)head * p.d + j] = v0;
+                    p.qk_raw[(size_t)head * p.d + j + hd] = v1;
+                } else {
+                    if (head < p.Hq + p.Hkv) {
+                        const float r0 = v0 * ea - v1 * eb, r1 = v1 * ea + v0 * eb;
+                        v0 = r0;
+                        v1 = r1;
+                    }
+                    if (head < p.Hq) {
+                        p.out[(size_t)head * p.d + j] = v0;
+                        p.out[(size_t)head * p.d + j + hd] = v1;
+                    } else {
+                        const int req = p.row_req ? p.row_req[0] : 0;
+                        const bool is_v = head >= p.Hq + p.Hkv;
+                        const int kh = head - p.Hq - (is_v ? p.Hkv : 0);
+                        uint16_t* row =
+                            reinterpret_cast<uint16_t*>(kv_row(p.kv, req, pos, is_v ? 1 : 0, kh, p.Hkv, p.d));
+                        row[j] = f2bf(v0);
+                        row[j + hd] = f2bf(v1);
+                    }
+                }
+            }
+        }
+        if (first + tpp < n_tiles) sync_consumers();  // the partial sums are rewritten by the next pass
+    }
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encoder() {
     static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
         void* f = nullptr;
@@ -527,7 +774,35 @@ cudaError_t launch_batch(const GemvParams& p, cudaStream_t st, bool pdl, int* nb
                : launch_batch_t<EPI, 8, false>(m0, m1, p, blocks, st, pdl);
 }
 
+template <int EPI>
+cudaError_t launch_ring(const GemvParams& p, cudaStream_t st, bool pdl) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    constexpr int UPT = TileUnits<EPI>::U;
+    const int tiles = (p.n_units + UPT - 1) / UPT, per = (tiles + sms - 1) / sms;
+    const int blocks = (tiles + per - 1) / per;
+    const uint64_t rows = EPI == EPI_QKV ? 2ull * p.n_units : (uint64_t)p.n_units;
+    CUtensorMap m0{}, m1{};
+    e = make_map(&m0, p.w0, rows, p.K);
+    if (e == cudaSuccess && EPI == EPI_SWIGLU) e = make_map(&m1, p.w1, rows, p.K);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(gemv_ring_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingSmem);
+    if (e != cudaSuccess) return e;
+    return launch_k(gemv_ring_kernel<EPI>, dim3(blocks), dim3(kRThreads), kRingSmem, st, pdl, m0, m1, p);
+}
+
 }  // namespace
+
+cudaError_t launch_gemv_ring(int epi, const GemvParams& p, cudaStream_t st, bool pdl) {
+    switch (epi) {
+        case EPI_QKV: return launch_ring<EPI_QKV>(p, st, pdl);
+        case EPI_RESID: return launch_ring<EPI_RESID>(p, st, pdl);
+        case EPI_SWIGLU: return launch_ring<EPI_SWIGLU>(p, st, pdl);
+        default: return cudaErrorInvalidValue;
+    }
+}
 
 cudaError_t launch_gemv_batch(int epi, const GemvParams& p, cudaStream_t st, bool pdl, int* nblocks_out) {
     switch (epi) {

@@ -1107,7 +1107,7 @@ struct loip_ctx {
                                     fixed_ptr<float>(fx.attn_scratch), o, false, s, pdl(), cfg.max_batch, true);
         });
         if (e != cudaSuccess) return cuda_fail(e, "attention kernel");
-        e = timed(2, s, [&] { return launch_resid_gemv(o, wo, B, H, qd, x, s, pdl(), host_a, true); });
+        e = timed(2, s, [&] { return launch_resid_gemv(o, wo, B, H, qd, x, s, pdl(), host_a); });
         if (e != cudaSuccess) return cuda_fail(e, "o-proj kernel");
         e = timed(3, s, [&] {
             return launch_gate_up(x, g_mlp, wg, wu, B, H, F, desc.rms_eps, a, s, pdl(), host_m);
@@ -2610,7 +2610,7 @@ extern "C" int loip_k_attention_tc_status(void) {
 extern "C" int loip_k_oproj(const float* o, const uint16_t* wo, int32_t B, int32_t H, int32_t K, float* x,
                             void* stream) {
     if (!o || !wo || !x || B < 1 || B > 8 || K % 8 || H < 1 || !al16(wo) || !al16(o)) return LOIP_ERR_INVALID;
-    return cerr(launch_resid_gemv(o, wo, B, H, K, x, (cudaStream_t)stream, false, false, true));
+    return cerr(launch_resid_gemv(o, wo, B, H, K, x, (cudaStream_t)stream));
 }
 
 extern "C" int loip_k_gate_up(const float* x, const uint16_t* g, const uint16_t* wg, const uint16_t* wu, int32_t B,

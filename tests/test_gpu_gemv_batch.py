@@ -1,6 +1,7 @@
 """The projections of 2 to 8 rows (three-part bf16 activations on the tensor
-cores) at the sizes where their tiling can go wrong, against the oracle within
-the a-priori fp32 summation bound, and their behaviour on infinities and NaN."""
+cores) and of one row (a ring of bulk copies) at the sizes where their tiling can
+go wrong, against the oracle within the a-priori fp32 summation bound, and their
+behaviour on infinities and NaN."""
 import numpy as np
 import pytest
 
@@ -22,7 +23,8 @@ def L():
 # (tensor-map loads or 16-byte copies); N: fewer rows than a tile, uneven ranges
 # per block, several passes of eight tiles (> 152 x 128 rows)
 @pytest.mark.parametrize("B,N,K", [(2, 1, 8), (8, 17, 64), (3, 4096, 512), (8, 300, 520), (5, 2433, 576),
-                                   (2, 1000, 1544), (8, 20000, 72), (4, 39000, 64)])
+                                   (2, 1000, 1544), (8, 20000, 72), (4, 39000, 64),
+                                   (1, 401, 10816), (1, 2433, 1984), (1, 66000, 64)])
 def test_resid_tiles(L, orc, B, N, K):
     a = inputs.normal_f32(3 * K + N, (B, K), 0.7)
     x0 = inputs.normal_f32(N, (B, N), 1.0)
@@ -38,7 +40,8 @@ def test_resid_tiles(L, orc, B, N, K):
 
 
 # the query / key / value ranges of a block begin and end inside a head
-@pytest.mark.parametrize("B,H,Hq,Hkv,d", [(2, 576, 40, 40, 128), (8, 200, 24, 3, 64), (5, 1024, 64, 8, 128)])
+@pytest.mark.parametrize("B,H,Hq,Hkv,d", [(2, 576, 40, 40, 128), (8, 200, 24, 3, 64), (5, 1024, 64, 8, 128),
+                                          (1, 576, 40, 40, 128), (1, 448, 72, 72, 64)])
 def test_qkv_ranges(L, orc, B, H, Hq, Hkv, d):
     import torch
     P, eps, theta = 64, 1e-5, 10000.0
