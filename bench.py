@@ -43,17 +43,17 @@ RUN_CLASS = 12  # kernel-timing class of the persistent layer-run kernel
 UNPACK_CLASS = 13  # kernel-timing class of the unpack of packed streamed chunks
 
 # DRAM bytes (read + write) per launch of the gate/up SwiGLU GEMV at batch 1
-# (the persistent kernel, at the 70B and the 8B shape), from an
+# (the ring kernel, at the 70B and the 8B shape), from an
 # ncu capture of the kernel microbenchmark on the model's shape (the
 # gate/up traffic summary among the ncu summaries has the commands).  They describe the
-# kernel source they were taken on: when the decode kernels' source no longer
+# kernel source they were taken on: when that source no longer
 # has this hash the figure is reported as null.
-GATE_UP_TRAFFIC = {"llama3-70b": 939_745_536, "llama3-8b": 235_113_984}
-GATE_UP_TRAFFIC_SRC = "a9c8cc3dcd122fa3d70d3d4bfa641301f6e3cb4caa4123b2fbe05cc51713aadc"
+GATE_UP_TRAFFIC = {"llama3-70b": 942_714_112, "llama3-8b": 237_965_824}
+GATE_UP_TRAFFIC_SRC = "75014321fbd7a30055db6db63f2cfe240a12c4592af60555c39b97acaa6dcfa8"
 
 
 def gate_up_traffic(model, batch):
-    src = os.path.join(ROOT, "paper_2512_21835_gb300", "csrc", "decode.cu")
+    src = os.path.join(ROOT, "paper_2512_21835_gb300", "csrc", "gemv_batch.cu")
     if batch != 1 or GATE_UP_TRAFFIC.get(model) is None:
         return None
     with open(src, "rb") as f:
@@ -65,8 +65,8 @@ def gate_up_traffic(model, batch):
 # DRAM bytes (read + write) of the unpack kernel per algorithmic byte (packed
 # chunk read + words written), from an ncu capture of the kernel microbenchmark
 # (one 70B layer's worth of words); valid while pack.cu has this hash.
-UNPACK_TRAFFIC_RATIO = 0.98081  # 2,858,692,352 B over 2,914,572,800 algorithmic (writes still in L2 at exit)
-UNPACK_TRAFFIC_SRC = "81016257b8e042a51f9c66df25f58d4d6acaf321fe224edfe44208a78c66e2dd"
+UNPACK_TRAFFIC_RATIO = 0.98086  # 2,858,798,336 B over 2,914,572,800 algorithmic (writes still in L2 at exit)
+UNPACK_TRAFFIC_SRC = "5a7ce38dc73850101a58d42b1c5e6b9eeae457b91dd1e67b3f46d9656c87fdb8"
 
 
 def unpack_traffic(bytes_per_launch):
